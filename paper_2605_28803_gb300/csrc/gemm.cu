@@ -31,7 +31,7 @@ cudaError_t launch_grouped(const GemmArgs& a) {
 // parts, 56.0 us against 53.9 whole) and 14500 for pairs (256-wide tiles in 2 parts, 45.2 us).
 enum class TileShape { kSingle128, kSingle256, kPair128, kPair256 };
 
-TileShape token_major_shape(const GemmArgs& a, int* parts) {
+TileShape token_major_shape(const GemmArgs& a, int* parts, long* estimate = nullptr) {
   const long nkb = a.K / kBK, sms = a.num_sms, npairs = a.num_sms / 2;
   const long t1 = (a.M + kBM - 1) / kBM, t2 = (a.M + 2 * kBM - 1) / (2 * kBM);
   const long n128 = a.gated ? 0 : (a.N + 127) / 128, n256 = (a.N + 255) / 256;
@@ -73,11 +73,32 @@ TileShape token_major_shape(const GemmArgs& a, int* parts) {
     consider(TileShape::kPair256, est(t2 * n256, npairs, 3800, 2900, 375, 256, 2, &q));
     if (n128) consider(TileShape::kPair128, est(t2 * n128, npairs, 3900, 1000, 351, 128, 2, &q));
   }
+  if (estimate) *estimate = t;
   return best;
+}
+
+// Whether the kernel with the weights in TMEM takes the launch, with its plan.  From K = 768 it was faster than the
+// token-major kernel at every shape measured (M 129-8192 and gated M 5-128, N 16-32768: 1.05 to 2.8 times); below, the
+// estimates decide.  Up to 128 tokens a layer that is not gated keeps the weight-major kernel: alone the other is faster
+// from K N = 2^21 or so, but between the small kernels of a chain it is not (the action head's step at 50 tokens: 240
+// against 221 us), as its pairs fill the SMs' shared memory and TMEM and so start late.
+bool take_tmem(const GemmArgs& a, int* bn, int* parts) {
+  if (a.num_sms < 2 || (!a.gated && a.M <= 128)) return false;
+  const long t = gemm_tmem_plan(a, bn, parts);
+  if (a.K >= 768) return true;
+  int unused = 1;
+  long old = 0;
+  token_major_shape(a, &unused, &old);
+  if (a.gated && old < 6900) old = 6900;  // a gated tile's epilogue outlasts a few k-blocks
+  return t < old;
 }
 
 template <int kX, typename OutT>
 cudaError_t launch_out(const GemmArgs& a) {
+  if constexpr (kX >= 1) {
+    int bn = 0, parts = 1;
+    if (take_tmem(a, &bn, &parts)) return launch_gemm_tmem(a, bn, parts);
+  }
   if (a.gated || a.M > 128) {
     if constexpr (kX == 2) {
       // 8-bit activation planes: single CTAs; tile width by waves x tile width

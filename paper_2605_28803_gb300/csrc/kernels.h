@@ -106,6 +106,14 @@ cudaError_t launch_gemm_w4a4(const GemmArgs& a);
 // units per tile (1 = whole tiles).
 int token_major_plan(const GemmArgs& a, int* parts);
 
+// The GEMM on CTA pairs with the expanded weights in TMEM (gemm_tmem.cu): operand-byte activations (x_bytes 1 or 2), one
+// scale per row, gated or not.  gemm_tmem_plan (host logic only) picks its tile width *bn (tokens, a multiple of 32) and
+// *parts, the work units per tile, and returns the estimated time in ns.  The outputs are the other kernels', bit for bit.
+long gemm_tmem_plan(const GemmArgs& a, int* bn, int* parts);
+cudaError_t launch_gemm_tmem(const GemmArgs& a, int bn, int parts);
+cudaError_t read_and_clear_error_word_tmem(unsigned int* out, cudaStream_t stream);
+cudaError_t set_debug_hooks_tmem(unsigned long long wait_limit_ns, int hold_loads);
+
 // The one-launch linear for a small batch with a per-step scale (gemm_fused.cu): the weight-major
 // split-K GEMM whose CTAs rotate and quantise the activations themselves.  *launched is false
 // (and nothing was enqueued) when the shape is outside what it takes: M > 128, gated or grouped

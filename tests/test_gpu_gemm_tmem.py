@@ -1,0 +1,114 @@
+"""GPU parity of the GEMM on CTA pairs with the expanded weights in TMEM (csrc/gemm_tmem.cu; Sec. 4.2, Eq. 7).
+
+qvla_w4a4_linear's GEMM takes it for batches of more than 128 tokens and for gated layers from 5 (below K = 768 where it is
+estimated faster); qvla_gemm_w4a4 on the same codes, packed, runs the token-major kernel.  Every accumulation is exact and the epilogue is the same operations, so the outputs must be the
+same bits.  Shapes sit at the edges of its tiles: one k-block and odd counts of them (the last ring stage holds one), token
+counts around the tile widths, weight rows past 64-, 128- and 256-row boundaries, tiles in several waves, K split into work
+units, and gated layers from a few tokens.  With 8-bit codes the accumulators must be the oracle's integers."""
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import qvla_oracle as O
+from paper_2605_28803_gb300 import qvla as Q
+from tests import gpu_helpers as G
+
+pytestmark = pytest.mark.gpu
+
+_T = {"f16": torch.float16, "bf16": torch.bfloat16}
+_C = {"f16": Q.F16, "bf16": Q.BF16}
+
+
+def _layer(rng, N, K, had, dt, gated=False):
+    rows = 2 * N if gated else N
+    wq = rng.integers(0, 256, (rows, K // 2), dtype=np.uint8)
+    ws = (rng.uniform(0.5, 1.5, rows) / 64).astype(np.float32)
+    bias = rng.standard_normal(rows).astype(np.float32)
+    if gated:
+        return Q.qvla_layer_create_gated(N, K, had, _C[dt], _C[dt], wq[:N], ws[:N], wq[N:], ws[N:], bias[:N], bias[N:]), wq
+    return Q.qvla_layer_create(N, K, had, _C[dt], _C[dt], wq, ws, bias), wq
+
+
+def _both(layer, x, M, dt):
+    """The linear through its workspace, and the public halves on packed codes."""
+    nb = Q.qvla_linear_workspace_bytes(layer, M)
+    work = torch.full((nb,), 0xA5, dtype=torch.uint8, device=G.DEV)
+    y = torch.full((M, layer.N), float("nan"), dtype=_T[dt], device=G.DEV)
+    Q.qvla_linear_quantize(layer, x, M, -1, work, nb, G.stream())
+    Q.qvla_linear_gemm(layer, work, nb, M, y, G.stream())
+    xq = torch.empty(M, layer.K // 2, dtype=torch.uint8, device=G.DEV)
+    xs = torch.empty(M, dtype=torch.float32, device=G.DEV)
+    xsum = torch.empty(M, dtype=torch.int32, device=G.DEV)
+    ref = torch.full((M, layer.N), float("nan"), dtype=_T[dt], device=G.DEV)
+    Q.qvla_rotate_quantize(layer, x, M, -1, xq, xs, xsum, G.stream())
+    Q.qvla_gemm_w4a4(layer, xq, xs, xsum, M, ref, None, G.stream())
+    Q.qvla_check_device(G.stream())
+    return y, ref
+
+
+@pytest.mark.parametrize("M,K,N,dt", [
+    (129, 768, 16, "f16"), (160, 896, 272, "bf16"), (191, 1152, 528, "f16"), (192, 1024, 1040, "bf16"),
+    (193, 2176, 1552, "f16"), (385, 1152, 4096, "bf16"), (2500, 1024, 2560, "f16"), (1500, 128, 4112, "bf16"),
+    (150, 16384, 2048, "bf16"), (300, 16384, 2000, "f16"), (700, 16384, 1904, "bf16")])
+def test_equals_the_other_kernels_bit_for_bit(M, K, N, dt):
+    rng = np.random.default_rng(M * 7 + K + N)
+    layer, _ = _layer(rng, N, K, 128, dt)
+    x = torch.from_numpy(rng.standard_normal((M, K), dtype=np.float32)).to(_T[dt]).to(G.DEV)
+    y, ref = _both(layer, x, M, dt)
+    assert torch.equal(y, ref)
+    layer.close()
+
+
+@pytest.mark.parametrize("M,K,H,dt", [(5, 128, 128, "bf16"), (33, 640, 256, "f16"), (128, 1152, 384, "bf16"),
+                                      (130, 896, 384, "f16"), (816, 2048, 1024, "bf16"), (1000, 768, 8192, "f16")])
+def test_gated_equals_the_token_major_kernel(M, K, H, dt):
+    rng = np.random.default_rng(M + K + H)
+    layer, _ = _layer(rng, H, K, 64, dt, gated=True)
+    x = torch.from_numpy(rng.standard_normal((M, K), dtype=np.float32)).to(_T[dt]).to(G.DEV)
+    y, ref = _both(layer, x, M, dt)
+    assert torch.equal(y, ref)
+    layer.close()
+
+
+@pytest.mark.parametrize("M,K,N,gated", [(200, 1152, 272, False), (129, 128, 16, False), (77, 896, 256, True)])
+def test_eight_bit_codes_give_the_oracles_integers(M, K, N, gated):
+    rng = np.random.default_rng(M + K)
+    layer, wq = _layer(rng, N, K, 1, "f16", gated)
+    xq = rng.integers(-127, 128, (M, K)).astype(np.int8)
+    nb = Q.qvla_w4a8_workspace_bytes(layer, M)
+    work = torch.empty(nb, dtype=torch.uint8, device=G.DEV)
+    acc = torch.full((M, wq.shape[0]), -1, dtype=torch.int32, device=G.DEV)
+    y = torch.empty(M, N, dtype=torch.float16, device=G.DEV)
+    xs = torch.full((M,), 1e-4, dtype=torch.float32, device=G.DEV)
+    Q.qvla_gemm_w4a8(layer, torch.from_numpy(xq).to(G.DEV), xs, M, y, acc, work, nb, G.stream())
+    Q.qvla_check_device(G.stream())
+    assert np.array_equal(acc.cpu().numpy(), O.int_gemm(xq, O.unpack_int4(wq)))
+    layer.close()
+
+
+def test_a_wait_that_runs_out_reports_timeout_and_the_next_launch_is_clean():
+    """With the hook no copy is issued: every role's wait runs out, no MMA is issued, nothing is written, the kernel
+    returns; the next launch is bit-exact."""
+    rng = np.random.default_rng(3)
+    M, K, N = 200, 1024, 512
+    layer, _ = _layer(rng, N, K, 128, "f16")
+    x = torch.from_numpy(rng.standard_normal((M, K), dtype=np.float32)).half().to(G.DEV)
+    y0, ref = _both(layer, x, M, "f16")
+    assert torch.equal(y0, ref)
+    nb = Q.qvla_linear_workspace_bytes(layer, M)
+    work = torch.empty(nb, dtype=torch.uint8, device=G.DEV)
+    y = torch.full((M, N), float("nan"), dtype=torch.float16, device=G.DEV)
+    Q.qvla_debug_set_hooks(20_000_000, True)
+    try:
+        Q.qvla_w4a4_linear(layer, x, M, -1, y, work, nb, G.stream())
+        with pytest.raises(Q.QvlaError) as e:
+            Q.qvla_check_device(G.stream())
+        assert e.value.status == 6
+        assert torch.isnan(y).all().item()
+    finally:
+        Q.qvla_debug_set_hooks(0, False)
+    Q.qvla_check_device(G.stream())
+    y1, _ = _both(layer, x, M, "f16")
+    assert torch.equal(y1, y0)
+    layer.close()
