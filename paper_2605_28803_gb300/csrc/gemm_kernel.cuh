@@ -426,7 +426,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w4a4_kernel(const __grid_con
   __shared__ __align__(16) float s_wc[kSwap ? 1 : kBN];
   __shared__ __align__(16) float s_bs[kSwap ? 1 : kBN];
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = warp_index();
   const int lane = threadIdx.x & 31;
 
   const int tiles_a = (p.rows_a + (kPair ? 2 : 1) * kBM - 1) / ((kPair ? 2 : 1) * kBM);
@@ -556,7 +556,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w4a4_kernel(const __grid_con
 
   if (warp == kTmaWarp) {
     // ------------------------------------------------------------------ TMA loads of packed tiles
-    if (lane == 0) {
+    if (elect_one()) {
       if constexpr (!kFused) tma_prefetch_desc(kSwap ? &tmap_b : &tmap_a);  // the activations' map (the weights need none)
       // Weight-major orientation with operand-byte activations: the staging ring holds weights
       // only, which no earlier kernel writes, so the first stages are requested before waiting
@@ -698,67 +698,21 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w4a4_kernel(const __grid_con
     if constexpr (kFused) fused_prologue(kEpiWarps + (warp - kTmaWarp - 1));
   } else if (warp == kMmaWarp) {
     // ------------------------------------------------------------------ MMA issuer
-    if (kPair && lane == 0 && prank == 0) {
-      constexpr uint32_t kIdesc = idesc_e4m3_f32(2 * kBM, kBN);
-      int it = 0, tile_iter = 0;
-      bool ok = true;
-      for (int u = QVLA_UNIT0; u < nunits && ok; u += QVLA_NUNITS, ++tile_iter) {
-        int tile, ka, kz;
-        unit_range(u, tile, ka, kz);
-        (void)tile;
-        const int buf = tile_iter & 1;
-        const uint32_t aph = static_cast<uint32_t>(tile_iter >> 1) & 1u;
-        if (!mbar_wait(smem_u32(&bar_tempty[buf]), aph ^ 1u)) { ok = false; break; }
-        tc_fence_after();
-        const uint32_t d = tmem_base + static_cast<uint32_t>(buf * kBN);
-        for (int kb = ka; kb < kz; ++kb, ++it) {
-          const int s = it % C::kStages;
-          const uint32_t ph = static_cast<uint32_t>(it / C::kStages) & 1u;
-          if (!mbar_wait(smem_u32(&bar_full[s]), ph)) { ok = false; break; }
-          tc_fence_after();
-          const uint32_t sa = smem_u32(smem + s * C::kStage);
-          const uint32_t sb = sa + C::kTileA;
-#pragma unroll
-          for (int kk = 0; kk < kBK / 32; ++kk)
-            mma_e4m3_pair(d, smem_desc_sw128(sa + kk * 32), smem_desc_sw128(sb + kk * 32), kIdesc,
-                          (kb != ka || kk != 0) ? 1u : 0u);
-          mma_commit_pair(smem_u32(&bar_empty[s]), 3);  // both CTAs' stage s is free
-        }
-        if (!ok) break;
-        mma_commit_pair(smem_u32(&bar_tfull[buf]), 3);
-      }
-      mma_commit_pair(smem_u32(&bar_done), 1);
-      mbar_wait(smem_u32(&bar_done), 0);
-    } else if (kPair && lane == 0) {
-      // the peer's forwarder: once this CTA's converters have filled stage s, one arrival tells
-      // the leader (the converters themselves arrive locally)
-      int it = 0;
-      bool ok = true;
-      for (int u = QVLA_UNIT0; u < nunits && ok; u += QVLA_NUNITS) {
-        int tile, ka, kz;
-        unit_range(u, tile, ka, kz);
-        (void)tile;
-        for (int kb = ka; kb < kz; ++kb, ++it) {
-          const int s = it % C::kStages;
-          if (!mbar_wait(smem_u32(&bar_full[s]), static_cast<uint32_t>(it / C::kStages) & 1u)) { ok = false; break; }
-          mbar_arrive_peer(mapa_shared(smem_u32(&bar_full[s]), 0));
-        }
-      }
-    } else if (kPair) {
-      // the other lanes of a pair's MMA warp have no role
-    } else if (lane == 0 && kGroup) {
-      // one accumulator per scale group, alternating between the two buffers group by group
-      constexpr uint32_t kIdesc = idesc_e4m3_f32(kBM, kBN);
-      int it = 0, gi = 0;
-      bool ok = true;
-      const int gkb = p.gkb;
-      for (int tile = QVLA_UNIT0; tile < ntiles && ok; tile += QVLA_NUNITS) {
-        for (int kg = kb0; kg < kb1; kg += gkb, ++gi) {
-          const int buf = gi & 1;
-          if (!mbar_wait(smem_u32(&bar_tempty[buf]), (static_cast<uint32_t>(gi >> 1) & 1u) ^ 1u)) { ok = false; break; }
+    if (kPair && prank == 0) {
+      if (elect_one()) {
+        constexpr uint32_t kIdesc = idesc_e4m3_f32(2 * kBM, kBN);
+        int it = 0, tile_iter = 0;
+        bool ok = true;
+        for (int u = QVLA_UNIT0; u < nunits && ok; u += QVLA_NUNITS, ++tile_iter) {
+          int tile, ka, kz;
+          unit_range(u, tile, ka, kz);
+          (void)tile;
+          const int buf = tile_iter & 1;
+          const uint32_t aph = static_cast<uint32_t>(tile_iter >> 1) & 1u;
+          if (!mbar_wait(smem_u32(&bar_tempty[buf]), aph ^ 1u)) { ok = false; break; }
           tc_fence_after();
           const uint32_t d = tmem_base + static_cast<uint32_t>(buf * kBN);
-          for (int q = 0; q < gkb; ++q, ++it) {
+          for (int kb = ka; kb < kz; ++kb, ++it) {
             const int s = it % C::kStages;
             const uint32_t ph = static_cast<uint32_t>(it / C::kStages) & 1u;
             if (!mbar_wait(smem_u32(&bar_full[s]), ph)) { ok = false; break; }
@@ -767,16 +721,66 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w4a4_kernel(const __grid_con
             const uint32_t sb = sa + C::kTileA;
 #pragma unroll
             for (int kk = 0; kk < kBK / 32; ++kk)
-              mma_e4m3(d, smem_desc_sw128(sa + kk * 32), smem_desc_sw128(sb + kk * 32), kIdesc, (q != 0 || kk != 0) ? 1u : 0u);
-            mma_commit(smem_u32(&bar_empty[s]));
+              mma_e4m3_pair(d, smem_desc_sw128(sa + kk * 32), smem_desc_sw128(sb + kk * 32), kIdesc,
+                            (kb != ka || kk != 0) ? 1u : 0u);
+            mma_commit_pair(smem_u32(&bar_empty[s]), 3);  // both CTAs' stage s is free
           }
           if (!ok) break;
-          mma_commit(smem_u32(&bar_tfull[buf]));
+          mma_commit_pair(smem_u32(&bar_tfull[buf]), 3);
+        }
+        mma_commit_pair(smem_u32(&bar_done), 1);
+        mbar_wait(smem_u32(&bar_done), 0);
+      }
+    } else if (kPair) {
+      if (elect_one()) {
+        // the peer's forwarder: once this CTA's converters have filled stage s, one arrival tells
+        // the leader (the converters themselves arrive locally)
+        int it = 0;
+        bool ok = true;
+        for (int u = QVLA_UNIT0; u < nunits && ok; u += QVLA_NUNITS) {
+          int tile, ka, kz;
+          unit_range(u, tile, ka, kz);
+          (void)tile;
+          for (int kb = ka; kb < kz; ++kb, ++it) {
+            const int s = it % C::kStages;
+            if (!mbar_wait(smem_u32(&bar_full[s]), static_cast<uint32_t>(it / C::kStages) & 1u)) { ok = false; break; }
+            mbar_arrive_peer(mapa_shared(smem_u32(&bar_full[s]), 0));
+          }
         }
       }
-      mma_commit(smem_u32(&bar_done));
-      mbar_wait(smem_u32(&bar_done), 0);
-    } else if (lane == 0) {
+    } else if (kGroup) {
+      if (elect_one()) {
+        // one accumulator per scale group, alternating between the two buffers group by group
+        constexpr uint32_t kIdesc = idesc_e4m3_f32(kBM, kBN);
+        int it = 0, gi = 0;
+        bool ok = true;
+        const int gkb = p.gkb;
+        for (int tile = QVLA_UNIT0; tile < ntiles && ok; tile += QVLA_NUNITS) {
+          for (int kg = kb0; kg < kb1; kg += gkb, ++gi) {
+            const int buf = gi & 1;
+            if (!mbar_wait(smem_u32(&bar_tempty[buf]), (static_cast<uint32_t>(gi >> 1) & 1u) ^ 1u)) { ok = false; break; }
+            tc_fence_after();
+            const uint32_t d = tmem_base + static_cast<uint32_t>(buf * kBN);
+            for (int q = 0; q < gkb; ++q, ++it) {
+              const int s = it % C::kStages;
+              const uint32_t ph = static_cast<uint32_t>(it / C::kStages) & 1u;
+              if (!mbar_wait(smem_u32(&bar_full[s]), ph)) { ok = false; break; }
+              tc_fence_after();
+              const uint32_t sa = smem_u32(smem + s * C::kStage);
+              const uint32_t sb = sa + C::kTileA;
+#pragma unroll
+              for (int kk = 0; kk < kBK / 32; ++kk)
+                mma_e4m3(d, smem_desc_sw128(sa + kk * 32), smem_desc_sw128(sb + kk * 32), kIdesc, (q != 0 || kk != 0) ? 1u : 0u);
+              mma_commit(smem_u32(&bar_empty[s]));
+            }
+            if (!ok) break;
+            mma_commit(smem_u32(&bar_tfull[buf]));
+          }
+        }
+        mma_commit(smem_u32(&bar_done));
+        mbar_wait(smem_u32(&bar_done), 0);
+      }
+    } else if (elect_one()) {
       constexpr uint32_t kIdesc = idesc_e4m3_f32(kBM, kBN);
       int it = 0, tile_iter = 0;
       bool ok = true;
