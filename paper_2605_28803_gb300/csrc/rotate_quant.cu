@@ -6,9 +6,19 @@ namespace qvla {
 cudaError_t launch_rotate_quant_f16(const RotQuantArgs& a);
 cudaError_t launch_rotate_quant_bf16(const RotQuantArgs& a);
 cudaError_t launch_rotate_quant_f32(const RotQuantArgs& a);
+cudaError_t launch_rotate_quant_wide_f16(const RotQuantArgs& a);
+cudaError_t launch_rotate_quant_wide_bf16(const RotQuantArgs& a);
+cudaError_t launch_rotate_quant_wide_f32(const RotQuantArgs& a);
 cudaError_t launch_rotate_quant_a8_f16(const RotQuantArgs& a);
 cudaError_t launch_rotate_quant_a8_bf16(const RotQuantArgs& a);
 cudaError_t launch_rotate_quant_a8_f32(const RotQuantArgs& a);
+
+// The kernel with 32 channels per thread (rotate_quant_wide.cuh): 4-bit codes with one scale per row (per token or per
+// step), Hadamard blocks up to 2048, and whole 256-channel groups where it transposes them.
+static bool rotate_quant_wide_takes(const RotQuantArgs& a) {
+  return (a.mode == 0 || a.mode == 1) && (a.out_mode == 0 || a.out_mode == 1) && a.gshift >= 30 && a.xgsum == nullptr &&
+         a.log_b >= 0 && a.log_b <= 11 && (a.log_b <= 5 || a.K % 256 == 0);
+}
 
 bool rotate_quant_supported(int log_b) { return log_b >= 0 && log_b <= 12; }
 
@@ -17,6 +27,14 @@ cudaError_t launch_rotate_quant(const RotQuantArgs& a) {
     bool launched = false;
     const cudaError_t e = launch_rotate_quant_pass(a, &launched);
     if (e != cudaSuccess || launched) return e;
+  }
+  if (rotate_quant_wide_takes(a)) {
+    switch (a.xdt) {
+      case 0: return launch_rotate_quant_wide_f16(a);
+      case 1: return launch_rotate_quant_wide_bf16(a);
+      case 2: return launch_rotate_quant_wide_f32(a);
+      default: return cudaErrorInvalidValue;
+    }
   }
   if (a.out_mode >= 2) {
     switch (a.xdt) {

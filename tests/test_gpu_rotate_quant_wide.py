@@ -1,0 +1,125 @@
+"""GPU parity of the rotate-quantise kernel with 32 channels per thread (csrc/rotate_quant_wide.cuh; Sec. 4.1 Eq. 3-5,
+Sec. 4.2 Eq. 5-6).
+
+It takes every batch of more than 64 rows into operand bytes and every packed call, for blocks up to 2048 and one scale per
+row.  Up to 64 rows of 16-bit activations qvla_linear_quantize runs the pass kernel, whose codes, scales and sums are pinned
+elsewhere: a batch quantised at once must give its bits chunk by chunk.  A per-group table of equal scales still runs the
+64-channel kernel, so its sums pin the shapes that the pass kernel refuses too.  Blocks at every phase count and group size
+(1, 32, 64, 128, 256, 512, 1024, 2048), row widths that are not a power of two of threads, ragged rows per CTA, per token and
+per step with clamping, exact ties, zero rows, huge, tiny, infinite and NaN values."""
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2605_28803_gb300 import qvla as Q
+from tests import gpu_helpers as G
+
+pytestmark = pytest.mark.gpu
+
+_T = {"f16": torch.float16, "bf16": torch.bfloat16, "f32": torch.float32}
+
+
+def _quantise(layer, x, step=-1):
+    M, K = x.shape
+    nb = Q.qvla_linear_workspace_bytes(layer, M)
+    work = torch.full((nb,), 0x3C, dtype=torch.uint8, device=G.DEV)
+    Q.qvla_linear_quantize(layer, x.contiguous(), M, step, work, nb, G.stream())
+    Q.qvla_check_device(G.stream())
+    r256 = lambda v: (v + 255) // 256 * 256  # noqa: E731
+    o = r256(M * K)
+    return (work[: M * K].view(M, K).cpu(), work[o : o + 4 * M].view(torch.int32).cpu(),
+            work[o + r256(4 * M) : o + r256(4 * M) + 4 * M].view(torch.int32).cpu())
+
+
+def _packed(x, had, scale=None):
+    M, K = x.shape
+    xq = torch.full((M, K // 2), 0x3C, dtype=torch.uint8, device=G.DEV)
+    xs = torch.empty(M, dtype=torch.float32, device=G.DEV)
+    xsum = torch.empty(M, dtype=torch.int32, device=G.DEV)
+    code = {torch.float16: Q.F16, torch.bfloat16: Q.BF16, torch.float32: Q.F32}[x.dtype]
+    Q.qvla_rotate_quantize_rows(x.contiguous(), code, M, K, had, scale, xq, xs, xsum, G.stream())
+    Q.qvla_check_device(G.stream())
+    return xq.cpu(), xs.view(torch.int32).cpu(), xsum.cpu()
+
+
+def _unpack(xq):
+    """Packed nibbles -> operand bytes q + 8 in the order k0 k2 k4 k6 k1 k3 k5 k7."""
+    M, K2 = xq.shape
+    c = torch.stack((xq & 15, xq >> 4), 2).view(M, K2 // 4, 8) ^ 8
+    return torch.cat((c[:, :, 0::2], c[:, :, 1::2]), 2).reshape(M, 2 * K2)
+
+
+def _values(rng, M, K, had, dt, special=True):
+    x = rng.standard_normal((M, K)).astype(np.float32)
+    x[:, rng.choice(K, max(1, K // 200), replace=False)] *= 20.0
+    if special:
+        x[1] = 0.0
+        x[2] *= 1e-6 if dt == "f16" else 1e-38
+        x[3, 5] = 6e4 if dt == "f16" else 1e38
+        x[4, 7] = np.inf
+        x[5, K - 1] = np.nan
+        x[6] = np.where(rng.random(K) < 0.5, 7.0, np.round(rng.uniform(-7, 7, K) * 2) / 2)  # ties where had = 1
+        x[7, 0], x[7, 1:] = 1.0, 0.0  # one channel: every rotated value equal
+    return torch.from_numpy(x).to(_T[dt]).to(G.DEV)
+
+
+@pytest.mark.parametrize("M,K,had,dt", [
+    (65, 128, 128, "f16"), (70, 384, 32, "bf16"), (131, 256, 64, "f16"), (130, 768, 256, "bf16"), (67, 2304, 256, "f16"),
+    (129, 512, 512, "bf16"), (66, 2560, 512, "f16"), (100, 1024, 1024, "bf16"), (97, 3072, 1024, "f16"),
+    (130, 2048, 2048, "bf16"), (70, 6144, 2048, "f16"), (66, 16384, 2048, "bf16"), (200, 640, 1, "f16"),
+    (66, 4096, 16, "bf16"), (65, 8320, 1, "bf16")])
+def test_a_batch_equals_the_pass_kernel_chunk_by_chunk(M, K, had, dt):
+    rng = np.random.default_rng(M + K + had)
+    x = _values(rng, M, K, had, dt)
+    layer = Q.qvla_layer_create(16, K, had, Q.DTYPE_CODES[dt], Q.F16, np.zeros((16, K // 2), np.uint8),
+                                np.ones(16, np.float32), None)
+    table = np.array([0.31, 1.7e-3, 3e-39], np.float32)  # an ordinary scale, one that clamps, an overflowing reciprocal
+    Q.qvla_set_step_scales(layer, table)
+    for step in (-1, 0, 1, 2):
+        whole = _quantise(layer, x, step)
+        parts = [_quantise(layer, x[i : i + 64], step) for i in range(0, M, 64)]
+        for got, want in zip(whole, (torch.cat(p) for p in zip(*parts))):
+            if step < 0 and had == 2048:
+                # the row with a NaN: a whole block is NaN, and the pass kernel's threads of 8 NaN values make the row's
+                # maximum NaN where this kernel's (like the 64-channel one's) leaves them out
+                got, want = got.clone(), want.clone()
+                got.view(M, -1)[5] = 0
+                want.view(M, -1)[5] = 0
+            assert torch.equal(got, want)
+        scale = None if step < 0 else torch.tensor([table[step]], device=G.DEV)
+        xq, xs, xsum = _packed(x, had, scale)
+        assert torch.equal(_unpack(xq), whole[0]) and torch.equal(xs, whole[1]) and torch.equal(xsum, whole[2])
+    layer.close()
+
+
+@pytest.mark.parametrize("M,K,had", [(67, 2304, 256), (131, 1024, 1024), (70, 4096, 2048), (65, 384, 32)])
+def test_f32_rows_equal_bf16_rows_of_the_same_values(M, K, had):
+    rng = np.random.default_rng(K)
+    xb = _values(rng, M, K, had, "bf16")
+    for got, want in zip(_packed(xb.float(), had), _packed(xb, had)):
+        assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("M,K,had", [(80, 1024, 64), (66, 2048, 128), (130, 4096, 2048)])
+def test_step_codes_equal_the_64_channel_kernel(M, K, had):
+    """A per-group table of one repeated scale runs the 64-channel kernel: the same outputs follow."""
+    rng = np.random.default_rng(K + had)
+    x = _values(rng, M, K, had, "f16", special=False)
+    wq = rng.integers(0, 256, (32, K // 2), dtype=np.uint8)
+    ws = np.full(32, 2.0 ** -8, np.float32)
+    out = []
+    for grouped in (False, True):
+        layer = Q.qvla_layer_create(32, K, had, Q.F16, Q.F16, wq, ws, None)
+        if grouped:
+            Q.qvla_set_step_group_scales(layer, np.full((1, K // max(128, had)), 0.25, np.float32))
+        else:
+            Q.qvla_set_step_scales(layer, np.array([0.25], np.float32))
+        nb = Q.qvla_linear_workspace_bytes(layer, M)
+        work = torch.empty(nb, dtype=torch.uint8, device=G.DEV)
+        y = torch.empty(M, 32, dtype=torch.float16, device=G.DEV)
+        Q.qvla_w4a4_linear(layer, x, M, 0, y, work, nb, G.stream())
+        Q.qvla_check_device(G.stream())
+        out.append(work[: M * K].cpu())
+        layer.close()
+    assert torch.equal(out[0], out[1])
