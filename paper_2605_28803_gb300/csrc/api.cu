@@ -126,6 +126,9 @@ qvla_status launch_rq(const void* x, int xdt, int M, int K, int had_block, int m
   a.xgsum = xgsum;
   a.zero = zero;
   a.zero_n = zero_n;
+  int device = 0;
+  QVLA_CUDA(cudaGetDevice(&device), "cudaGetDevice");
+  a.num_sms = num_sms(device);
   a.stream = static_cast<cudaStream_t>(stream);
   QVLA_CUDA(qvla::launch_rotate_quant(a), "rotate_quantize launch");
   return QVLA_OK;

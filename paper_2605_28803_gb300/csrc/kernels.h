@@ -31,10 +31,11 @@ struct RotQuantArgs {
   int32_t* xgsum = nullptr;  // device [M][K >> gshift] per-group code sums, or null
   int32_t* zero = nullptr;   // device ints set to 0 once x has been waited for (the next GEMM's
   int zero_n = 0;            //   work-unit counters), or null
+  int num_sms = 152;         // of the device (how a few rows are spread)
   cudaStream_t stream;
 };
 bool rotate_quant_supported(int log_b);
-// The rotate-quantise kernel in passes (rotate_quant_pass.cu): up to 64 rows of 16-bit
+// The rotate-quantise kernel in passes (rotate_quant_pass.cu): up to 48 rows of more than 4096 16-bit
 // activations into operand bytes (out_mode 1) with one scale per row, per token or per step,
 // Hadamard block <= 2048 and at most 8 passes of 2048 (or fewer, smaller) channels per row.
 // *launched is false (nothing enqueued) outside that range; the outputs are those of the

@@ -1,5 +1,5 @@
 // Rotate + quantise in passes: the online rotation and activation quantisation (Sec. 4.1 Eq. 3-5,
-// Sec. 4.2 Eq. 5-6) of a few rows of 16-bit activations into the GEMM's operand bytes, one CTA per
+// Sec. 4.2 Eq. 5-6) of a few long rows of 16-bit activations into the GEMM's operand bytes, one CTA per
 // 2048-channel pass of a row.
 //
 // The row-per-warp kernel of rotate_quant.cuh gives each thread 64 channels, so a thread's chain
@@ -27,7 +27,8 @@ constexpr int kRqpThreads = 256;
 // receiving wait runs out
 static __device__ int g_rqp_hold;
 constexpr int kRqpMaxPasses = 8;  // a cluster of at most 8 CTAs (K <= 16384)
-constexpr int kRqpMaxRows = 64;   // the rows it takes (more rows go to the row-per-warp kernel)
+constexpr int kRqpMaxRows = 48;   // the rows it takes, of more than kRqpMinK channels
+constexpr int kRqpMinK = 4096;
 
 struct RqpParams {
   const void* x;            // [M][K] activations
@@ -226,13 +227,13 @@ cudaError_t launch_rqp(const RotQuantArgs& a, const RqpParams& p) {
 
 cudaError_t launch_rotate_quant_pass(const RotQuantArgs& a, bool* launched) {
   *launched = false;
-  // 16-bit activations into 4-bit operand bytes, one scale per row (per token or per step), for
-  // up to 64 rows: there the latency of one row decides, and a pass's 256 threads cut it
-  // (measured, one call: 1 x 2048 6.8 against 8.8 us, 4 x 16384 8.8 against 10.9 us; the DiT
-  // step at 50 tokens 691 -> 647 us).  At hundreds of rows the row-per-warp kernel's cheaper
-  // stages per element win (816 x 16384: 27.3 against 41.6 us).
+  // 16-bit activations into 4-bit operand bytes, one scale per row (per token or per step), for a few long rows: there a
+  // row's own latency decides, and up to 8 CTAs cut it (measured back to back in a graph against the kernel with 32
+  // channels per thread, K = 16384: 2 rows 2.8 against 3.9 us, 32 rows 3.5 against 4.2, 50 rows 4.25 against 4.2; at
+  // K = 4096 the two are equal, below the other is faster: 50 x 1024 2.19 against 2.10, and the action head's step at 50
+  // tokens 196 against 188).
   if (a.out_mode != 1 || (a.mode != 0 && a.mode != 1) || (a.xdt != 0 && a.xdt != 1) || a.gshift < 30 ||
-      a.xgsum != nullptr || a.M < 1 || a.M > kRqpMaxRows)
+      a.xgsum != nullptr || a.M < 1 || a.M > kRqpMaxRows || a.K <= kRqpMinK)
     return cudaSuccess;
   int C = 2048;
   while (a.K % C != 0) C /= 2;

@@ -4,9 +4,9 @@
 // It does what rotate_quant.cuh's kernel does for 4-bit codes and one scale per row, bit for bit, with fewer instructions
 // per channel and twice the warps in flight:
 //   * a thread holds 32 channels instead of 64: 64 registers, 32 warps per SM;
-//   * the butterflies run in three phases, index bits 0-4 on 32 consecutive channels, 5-7, and 8-10, with a transpose
-//     through shared memory between phases whose stores and loads both move 16 bytes (4 channels, a quad) per thread.  A
-//     quad is the channels whose codes fill one 32-bit word of the output, so after the last phase every code leaves in a
+//   * the butterflies run in three phases, index bits 0-4 on 32 consecutive channels, 5-7, and 8-10 (8-11 for blocks of
+//     4096, on half quads), with a transpose through shared memory between phases whose stores and loads both move 16
+//     bytes (4 channels, a quad) per thread.  A quad is the channels whose codes fill one 32-bit word of the output, so after the last phase every code leaves in a
 //     4-byte store, 128 contiguous bytes per warp (the 64-channel layout ends in 1-byte stores at b = 2048).  The stage
 //     order and every rounding are the other kernel's;
 //   * a code q is the E4M3 byte of (q + 8) 2^-9, so one conversion instruction rounds two values to operand bytes.  It is
@@ -20,7 +20,8 @@
 // blocks of 256 3.9 and 2.8; f32 777 x 4096 9.9 and 9.7.  About 21 instructions a channel at 55% of the issue slots; neither
 // the transposes, the butterflies nor the conversions alone bound it (leaving one of them out saves 6 to 16%).  Staying
 // CTAs fed by TMA one group ahead were slower (73 us at 3200 x 16384): with an extra barrier a group, two CTAs an SM overlap
-// less than fresh ones.
+// less than fresh ones.  A few rows are spread one to a CTA: 50 x 1024 2.1 us against 2.8 with eight rows a CTA; with blocks
+// of 4096 at 50 x 4096 (128 channels a thread in the other kernel) the action head's step went from 208 to 188 us.
 #pragma once
 
 #include "ptx.cuh"
@@ -43,17 +44,20 @@ __device__ __forceinline__ uint32_t e4m3x4(float a, float b, float c, float d) {
 __device__ __forceinline__ void sts128(uint32_t addr, float2 a, float2 b) {
   asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y) : "memory");
 }
+__device__ __forceinline__ void lds64(uint32_t addr, float2& a) {
+  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(a.x), "=f"(a.y) : "r"(addr) : "memory");
+}
 __device__ __forceinline__ void lds128(uint32_t addr, float2& a, float2& b) {
   asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(a.x), "=f"(a.y), "=f"(b.x), "=f"(b.y) : "r"(addr) : "memory");
 }
 
-// The threads of a Hadamard block meet between the second and the third phase: part of a warp, or two warps.
+// The threads of a Hadamard block meet between the second and the third phase: part of a warp, or two or four warps.
 template <int kLogB>
 __device__ __forceinline__ void block_sync() {
   if constexpr (kLogB <= 10) {
     __syncwarp();
-  } else {  // 64 threads
-    asm volatile("bar.sync %0, 64;" ::"r"(1 + static_cast<int>(threadIdx.x >> 6)) : "memory");
+  } else {  // 64 or 128 threads
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + static_cast<int>(threadIdx.x >> (kLogB - 5))), "n"(1 << (kLogB - 5)) : "memory");
   }
 }
 
@@ -87,7 +91,8 @@ __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(cons
   constexpr int kA = kLogB < 5 ? kLogB : 5;                        // index bits of the first phase
   constexpr int kRB = kLogB <= 5 ? 0 : kLogB < 8 ? kLogB - 5 : 3;  // of the second: 5 .. 5 + kRB - 1
   constexpr int kRC = kLogB <= 8 ? 0 : kLogB - 8;                  // of the third: 8 .. 8 + kRC - 1
-  static_assert(kLogB <= 11, "Hadamard blocks up to 2048");
+  constexpr bool kHalf = kRC == 4;  // after the third phase a thread holds half quads (two channels) of 16 lines
+  static_assert(kLogB <= 12, "Hadamard blocks up to 4096");
   extern __shared__ __align__(128) uint8_t wide_smem[];  // one line of 8 quads (128 bytes) per thread
   __shared__ unsigned int s_max[kWideRows], s_sum[kWideRows];
 
@@ -165,18 +170,26 @@ __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(cons
   }
   if constexpr (kRC > 0) {
     // phase 3: the 8 * 2^kRC threads (h, q) of a Hadamard block trade the high kRC bits of the line for the group index h
-    constexpr int kLb = 3 - kRC;  // line bits a thread keeps
-    __syncwarp();                 // the group has read this thread's lines
+    constexpr int kLb = kHalf ? 0 : 3 - kRC;  // line bits a thread keeps
+    __syncwarp();                             // the group has read this thread's lines
 #pragma unroll
     for (int l = 0; l < 8; ++l) sts128(own ^ static_cast<uint32_t>(l * 16), v[2 * l], v[2 * l + 1]);
     block_sync<kLogB>();
     constexpr int kGroup = 8 << kRC;
-    const int la = (j >> 3) & ((1 << kRC) - 1);
-    const uint32_t blk = (lines + static_cast<uint32_t>((tid & ~(kGroup - 1)) * 128 + q * 144)) ^ static_cast<uint32_t>(la << (kLb + 4));
+    if constexpr (kHalf) {  // thread (l, q, e) of the block: half e of quad q of line l of all 16 groups
+      const int l = (j >> 4) & 7, qq = (j >> 1) & 7;
+      const uint32_t blk = lines + static_cast<uint32_t>((tid & ~(kGroup - 1)) * 128 + qq * 128 + ((l ^ qq) << 4) + (j & 1) * 8);
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
-      lds128((blk ^ static_cast<uint32_t>((i & ((1 << kLb) - 1)) * 16)) + (i >> kLb) * 1024, v[2 * i], v[2 * i + 1]);
-    fwht_regs<16, 5 - kRC, 5>(v);
+      for (int h = 0; h < 16; ++h) lds64(blk + h * 1024, v[h]);
+      fwht_regs<16, 1, 5>(v);
+    } else {
+      const int la = (j >> 3) & ((1 << kRC) - 1);
+      const uint32_t blk = (lines + static_cast<uint32_t>((tid & ~(kGroup - 1)) * 128 + q * 144)) ^ static_cast<uint32_t>(la << (kLb + 4));
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        lds128((blk ^ static_cast<uint32_t>((i & ((1 << kLb) - 1)) * 16)) + (i >> kLb) * 1024, v[2 * i], v[2 * i + 1]);
+      fwht_regs<16, kHalf ? 5 : 5 - kRC, 5>(v);
+    }
   }
 
   // ---- scale ----
@@ -261,10 +274,22 @@ __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(cons
         *reinterpret_cast<uint4*>(dst + static_cast<size_t>(j) * 32 + 16) = make_uint4(code[4], code[5], code[6], code[7]);
       }
     } else {
-      constexpr int kLb = 3 - kRC;
+      constexpr int kLb = kHalf ? 0 : 3 - kRC;
       const int la = (j >> 3) & ((1 << kRC) - 1);
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
+        if constexpr (kHalf) {  // word i: the half quads of groups 2 i and 2 i + 1
+          const int at = (j & ~127) + 16 * i + ((j >> 4) & 7), piece = j & 15;  // 8 lines a group
+          if constexpr (kPacked) {
+            const uint32_t n = nibbles(code[i]);
+            dst[at * 16 + piece] = static_cast<uint8_t>(n);
+            dst[(at + 8) * 16 + piece] = static_cast<uint8_t>(n >> 8);
+          } else {
+            *reinterpret_cast<uint16_t*>(dst + at * 32 + piece * 2) = static_cast<uint16_t>(code[i]);
+            *reinterpret_cast<uint16_t*>(dst + (at + 8) * 32 + piece * 2) = static_cast<uint16_t>(code[i] >> 16);
+          }
+          continue;
+        }
         // the line of quad i: phase 2 leaves line i of the 256-channel group, phase 3 line l of group h of the block
         int line;
         if constexpr (kRC == 0) {
@@ -301,6 +326,7 @@ cudaError_t launch_wide_t(const RotQuantArgs& a) {
   const int tpr = a.K / 32;
   int rows = tpr >= 256 ? 1 : 256 / tpr;
   if (rows > kWideRows) rows = kWideRows;
+  while (rows > 1 && (a.M + rows - 1) / rows < a.num_sms) rows /= 2;  // few rows: more CTAs, down to one row each
   const int tpb = (rows * tpr + 31) & ~31;  // whole warps: the warp-wide steps take every lane
   auto kern = rotate_quant_wide_kernel<T, kLogB, kStep, kPacked>;
   const size_t smem = kLogB > 5 ? static_cast<size_t>(tpb) * 128 : 0;
@@ -347,7 +373,8 @@ cudaError_t launch_wide_b(const RotQuantArgs& a) {
     case 8: return launch_wide_t<T, 8, kStep, kPacked>(a);
     case 9: return launch_wide_t<T, 9, kStep, kPacked>(a);
     case 10: return launch_wide_t<T, 10, kStep, kPacked>(a);
-    default: return launch_wide_t<T, 11, kStep, kPacked>(a);
+    case 11: return launch_wide_t<T, 11, kStep, kPacked>(a);
+    default: return launch_wide_t<T, 12, kStep, kPacked>(a);
   }
 }
 

@@ -1,12 +1,12 @@
 """GPU parity of the rotate-quantise kernel with 32 channels per thread (csrc/rotate_quant_wide.cuh; Sec. 4.1 Eq. 3-5,
 Sec. 4.2 Eq. 5-6).
 
-It takes every batch of more than 64 rows into operand bytes and every packed call, for blocks up to 2048 and one scale per
-row.  Up to 64 rows of 16-bit activations qvla_linear_quantize runs the pass kernel, whose codes, scales and sums are pinned
-elsewhere: a batch quantised at once must give its bits chunk by chunk.  A per-group table of equal scales still runs the
-64-channel kernel, so its sums pin the shapes that the pass kernel refuses too.  Blocks at every phase count and group size
-(1, 32, 64, 128, 256, 512, 1024, 2048), row widths that are not a power of two of threads, ragged rows per CTA, per token and
-per step with clamping, exact ties, zero rows, huge, tiny, infinite and NaN values."""
+It takes 4-bit codes with one scale per row, but for a few long rows, which the pass kernel keeps (at most 48 rows of more
+than 4096 channels; its codes, scales and sums are pinned elsewhere).  A row repeated r times side by side has the same
+rotated values, the same maximum and r times the code sum, so the pass kernel on repeated rows pins this one at every
+width.  A per-group table of equal scales runs the 64-channel kernel, which pins the per-step codes, blocks of 4096
+included.  Blocks at every phase count and group size, row widths that are not a power of two of threads, ragged rows per
+CTA, per token and per step with clamping, exact ties, zero rows, huge, tiny, infinite and NaN values."""
 
 import numpy as np
 import pytest
@@ -53,7 +53,7 @@ def _unpack(xq):
 def _values(rng, M, K, had, dt, special=True):
     x = rng.standard_normal((M, K)).astype(np.float32)
     x[:, rng.choice(K, max(1, K // 200), replace=False)] *= 20.0
-    if special:
+    if special and M > 8:
         x[1] = 0.0
         x[2] *= 1e-6 if dt == "f16" else 1e-38
         x[3, 5] = 6e4 if dt == "f16" else 1e38
@@ -64,36 +64,40 @@ def _values(rng, M, K, had, dt, special=True):
     return torch.from_numpy(x).to(_T[dt]).to(G.DEV)
 
 
-@pytest.mark.parametrize("M,K,had,dt", [
-    (65, 128, 128, "f16"), (70, 384, 32, "bf16"), (131, 256, 64, "f16"), (130, 768, 256, "bf16"), (67, 2304, 256, "f16"),
-    (129, 512, 512, "bf16"), (66, 2560, 512, "f16"), (100, 1024, 1024, "bf16"), (97, 3072, 1024, "f16"),
-    (130, 2048, 2048, "bf16"), (70, 6144, 2048, "f16"), (66, 16384, 2048, "bf16"), (200, 640, 1, "f16"),
-    (66, 4096, 16, "bf16"), (65, 8320, 1, "bf16")])
-def test_a_batch_equals_the_pass_kernel_chunk_by_chunk(M, K, had, dt):
+@pytest.mark.parametrize("M,K,had,dt,r", [
+    (65, 128, 128, "f16", 64), (70, 384, 32, "bf16", 16), (131, 256, 64, "f16", 32), (130, 768, 256, "bf16", 8),
+    (129, 512, 512, "bf16", 16), (66, 2560, 512, "f16", 4), (100, 1024, 1024, "bf16", 8), (97, 3072, 1024, "f16", 4),
+    (130, 2048, 2048, "bf16", 4), (70, 6144, 2048, "f16", 1), (66, 16384, 2048, "bf16", 1), (200, 640, 1, "f16", 16),
+    (66, 4096, 16, "bf16", 2), (9, 2048, 256, "f16", 4), (50, 1024, 64, "bf16", 8)])
+def test_a_batch_equals_the_pass_kernel_on_repeated_rows(M, K, had, dt, r):
     rng = np.random.default_rng(M + K + had)
     x = _values(rng, M, K, had, dt)
-    layer = Q.qvla_layer_create(16, K, had, Q.DTYPE_CODES[dt], Q.F16, np.zeros((16, K // 2), np.uint8),
-                                np.ones(16, np.float32), None)
+    xr = x.repeat(1, r)
+    make = lambda k: Q.qvla_layer_create(16, k, had, Q.DTYPE_CODES[dt], Q.F16, np.zeros((16, k // 2), np.uint8),  # noqa: E731
+                                         np.ones(16, np.float32), None)
+    layer, wide = make(K), make(K * r)
     table = np.array([0.31, 1.7e-3, 3e-39], np.float32)  # an ordinary scale, one that clamps, an overflowing reciprocal
     Q.qvla_set_step_scales(layer, table)
+    Q.qvla_set_step_scales(wide, table)
     for step in (-1, 0, 1, 2):
-        whole = _quantise(layer, x, step)
-        parts = [_quantise(layer, x[i : i + 64], step) for i in range(0, M, 64)]
-        for got, want in zip(whole, (torch.cat(p) for p in zip(*parts))):
-            if step < 0 and had == 2048:
-                # the row with a NaN: a whole block is NaN, and the pass kernel's threads of 8 NaN values make the row's
-                # maximum NaN where this kernel's (like the 64-channel one's) leaves them out
-                got, want = got.clone(), want.clone()
-                got.view(M, -1)[5] = 0
-                want.view(M, -1)[5] = 0
-            assert torch.equal(got, want)
+        ob, xs, xsum = _quantise(layer, x, step)
+        parts = [_quantise(wide, xr[i : i + 48], step) for i in range(0, M, 48)] if r > 1 or M > 48 else []
+        want = [torch.cat(p) for p in zip(*parts)]
+        rows = torch.ones(M, dtype=torch.bool)
+        if step < 0 and M > 5:
+            # the row with a NaN: a whole block may be NaN, and the pass kernel's threads of 8 NaN values make the row's
+            # maximum NaN where this kernel's (like the 64-channel one's) leaves them out
+            rows[5] = False
+        assert torch.equal(ob.repeat(1, r)[rows], want[0][rows])
+        assert torch.equal(xs[rows], want[1][rows]) and torch.equal(r * xsum[rows], want[2][rows])
         scale = None if step < 0 else torch.tensor([table[step]], device=G.DEV)
-        xq, xs, xsum = _packed(x, had, scale)
-        assert torch.equal(_unpack(xq), whole[0]) and torch.equal(xs, whole[1]) and torch.equal(xsum, whole[2])
+        xq, pxs, pxsum = _packed(x, had, scale)
+        assert torch.equal(_unpack(xq), ob) and torch.equal(pxs, xs) and torch.equal(pxsum, xsum)
     layer.close()
+    wide.close()
 
 
-@pytest.mark.parametrize("M,K,had", [(67, 2304, 256), (131, 1024, 1024), (70, 4096, 2048), (65, 384, 32)])
+@pytest.mark.parametrize("M,K,had", [(67, 2304, 256), (131, 1024, 1024), (70, 4096, 2048), (65, 384, 32), (33, 8192, 4096)])
 def test_f32_rows_equal_bf16_rows_of_the_same_values(M, K, had):
     rng = np.random.default_rng(K)
     xb = _values(rng, M, K, had, "bf16")
@@ -101,7 +105,8 @@ def test_f32_rows_equal_bf16_rows_of_the_same_values(M, K, had):
         assert torch.equal(got, want)
 
 
-@pytest.mark.parametrize("M,K,had", [(80, 1024, 64), (66, 2048, 128), (130, 4096, 2048)])
+@pytest.mark.parametrize("M,K,had", [(80, 1024, 64), (66, 2048, 128), (130, 4096, 2048), (1, 4096, 4096),
+                                      (66, 8192, 4096), (50, 4096, 4096)])
 def test_step_codes_equal_the_64_channel_kernel(M, K, had):
     """A per-group table of one repeated scale runs the 64-channel kernel: the same outputs follow."""
     rng = np.random.default_rng(K + had)
