@@ -14,10 +14,10 @@ cudaError_t launch_rotate_quant_a8_bf16(const RotQuantArgs& a);
 cudaError_t launch_rotate_quant_a8_f32(const RotQuantArgs& a);
 
 // The kernel with 32 channels per thread (rotate_quant_wide.cuh): 4-bit codes with one scale per row (per token or per
-// step), and whole 256-channel groups where it transposes them.
+// step).  K is a multiple of 128 and of the block, which is all that its groups of threads need.
 static bool rotate_quant_wide_takes(const RotQuantArgs& a) {
   return (a.mode == 0 || a.mode == 1) && (a.out_mode == 0 || a.out_mode == 1) && a.gshift >= 30 && a.xgsum == nullptr &&
-         a.log_b >= 0 && a.log_b <= 12 && (a.log_b <= 5 || a.K % 256 == 0);
+         a.log_b >= 0 && a.log_b <= 12;
 }
 
 bool rotate_quant_supported(int log_b) { return log_b >= 0 && log_b <= 12; }

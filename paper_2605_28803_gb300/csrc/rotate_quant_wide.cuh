@@ -4,8 +4,8 @@
 // It does what rotate_quant.cuh's kernel does for 4-bit codes and one scale per row, bit for bit, with fewer instructions
 // per channel and twice the warps in flight:
 //   * a thread holds 32 channels instead of 64: 64 registers, 32 warps per SM;
-//   * the butterflies run in three phases, index bits 0-4 on 32 consecutive channels, 5-7, and 8-10 (8-11 for blocks of
-//     4096, on half quads), with a transpose through shared memory between phases whose stores and loads both move 16
+//   * the butterflies run in three phases, index bits 0-4 on 32 consecutive channels, 5-7 (5-6 among 4 threads for blocks of
+//     64 and 128, whose rows need not be whole 256-channel groups), and 8-10 (8-11 for blocks of 4096, on half quads), with a transpose through shared memory between phases whose stores and loads both move 16
 //     bytes (4 channels, a quad) per thread.  A quad is the channels whose codes fill one 32-bit word of the output, so after the last phase every code leaves in a
 //     4-byte store, 128 contiguous bytes per warp (the 64-channel layout ends in 1-byte stores at b = 2048).  The stage
 //     order and every rounding are the other kernel's;
@@ -17,7 +17,8 @@
 //
 // Measured back to back in a graph, 64-channel kernel before and this one, us: 816 x 2048 bf16 5.9 and 4.8; 816 x 16384
 // 23.0 and 18.0; 3200 x 16384 f16 72.0 and 58.4 (2.7 TB/s of x and codes); 8192 x 2048 22.7 and 19.3; 201 x 2304 with
-// blocks of 256 3.9 and 2.8; f32 777 x 4096 9.9 and 9.7.  About 21 instructions a channel at 55% of the issue slots; neither
+// blocks of 256 3.9 and 2.8; f32 777 x 4096 9.9 and 9.7; blocks of 128: 3325 x 10112 47.3 and 32.0, 7761 x 2688 29.3 and 20.6,
+// 8192 x 384 8.6 and 5.2.  About 21 instructions a channel at 55% of the issue slots; neither
 // the transposes, the butterflies nor the conversions alone bound it (leaving one of them out saves 6 to 16%).  Staying
 // CTAs fed by TMA one group ahead were slower (73 us at 3200 x 16384): with an extra barrier a group, two CTAs an SM overlap
 // less than fresh ones.  A few rows are spread one to a CTA: 50 x 1024 2.1 us against 2.8 with eight rows a CTA; with blocks
@@ -91,6 +92,8 @@ __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(cons
   constexpr int kA = kLogB < 5 ? kLogB : 5;                        // index bits of the first phase
   constexpr int kRB = kLogB <= 5 ? 0 : kLogB < 8 ? kLogB - 5 : 3;  // of the second: 5 .. 5 + kRB - 1
   constexpr int kRC = kLogB <= 8 ? 0 : kLogB - 8;                  // of the third: 8 .. 8 + kRC - 1
+  // blocks of 64 and 128: the second phase trades among 4 threads, so that a row needs whole 128-channel groups only
+  constexpr bool kFour = kRB == 1 || kRB == 2;
   constexpr bool kHalf = kRC == 4;  // after the third phase a thread holds half quads (two channels) of 16 lines
   static_assert(kLogB <= 12, "Hadamard blocks up to 4096");
   extern __shared__ __align__(128) uint8_t wide_smem[];  // one line of 8 quads (128 bytes) per thread
@@ -102,6 +105,8 @@ __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(cons
   const int m = blockIdx.x * rpc + rloc;
   const bool active = rloc < rpc && m < M;
   const bool one_warp = tpr == 32;  // a row is a warp: no shared reduction
+  // a warp within one row reduces as a warp; else its groups of 4 threads (K is a multiple of 128), if whole
+  const bool row_warp = __shfl_sync(0xffffffffu, rloc, 0) == __shfl_sync(0xffffffffu, rloc, 31);
   if (tid < kWideRows) {
     s_max[tid] = 0u;
     s_sum[tid] = 0u;
@@ -158,7 +163,20 @@ __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(cons
   // quad i of line l lies at piece i ^ (l % 8) of the line's 128 bytes: stores and loads of 8 threads meet 8 pieces
   const uint32_t lines = smem_u32(wide_smem);
   const uint32_t own = lines + static_cast<uint32_t>(tid * 128 + q * 16);
-  if constexpr (kRB > 0) {
+  if constexpr (kFour) {
+    // phase 2: thread p of the 4 of a 128-channel group takes quads 2 p and 2 p + 1 of its lines.  Quad i of line l at piece
+    // i ^ s(l), s = 0 2 4 6 1 3 5 7 over 8 lines: the even pieces two groups read at a time fall on all eight
+    const int g = (tid >> 2) & 1, p = tid & 3;
+    const uint32_t line = lines + static_cast<uint32_t>(tid * 128 + (2 * p + g) * 16);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) sts128(line ^ static_cast<uint32_t>(i * 16), v[2 * i], v[2 * i + 1]);
+    __syncwarp();
+    const uint32_t grp = lines + static_cast<uint32_t>((tid & ~3) * 128 + ((2 * p) ^ g) * 16);
+#pragma unroll
+    for (int i = 0; i < 8; ++i)  // i = 2 l + e
+      lds128((grp ^ static_cast<uint32_t>(i * 16)) + (i >> 1) * 128, v[2 * i], v[2 * i + 1]);
+    fwht_regs<16, 3, 3 + kRB>(v);
+  } else if constexpr (kRB > 0) {
     // phase 2: the 8 threads of a 256-channel group trade quads for lines; line l of the group at thread l's place
 #pragma unroll
     for (int i = 0; i < 8; ++i) sts128(own ^ static_cast<uint32_t>(i * 16), v[2 * i], v[2 * i + 1]);
@@ -201,11 +219,13 @@ __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(cons
 #pragma unroll
     for (int i = 0; i < 16; ++i) w = fmaxf(w, fmaxf(fabsf(v[i].x), fabsf(v[i].y)));
     unsigned int wm = __float_as_uint(w);  // non-negative floats order as their bit patterns
-    if ((tpr & 31) == 0) {
+    if (row_warp) {
       wm = __reduce_max_sync(0xffffffffu, wm);
-      if (!one_warp && (tid & 31) == 0) atomicMax(&s_max[rloc], wm);
-    } else if (rloc < rpc) {
-      atomicMax(&s_max[rloc], wm);
+      if (!one_warp && (tid & 31) == 0 && rloc < rpc) atomicMax(&s_max[rloc], wm);
+    } else {
+      wm = max(wm, __shfl_xor_sync(0xffffffffu, wm, 1));
+      wm = max(wm, __shfl_xor_sync(0xffffffffu, wm, 2));
+      if ((tid & 3) == 0 && rloc < rpc) atomicMax(&s_max[rloc], wm);
     }
     if (!one_warp) {
       __syncthreads();
@@ -273,6 +293,16 @@ __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(cons
         *reinterpret_cast<uint4*>(dst + static_cast<size_t>(j) * 32) = make_uint4(code[0], code[1], code[2], code[3]);
         *reinterpret_cast<uint4*>(dst + static_cast<size_t>(j) * 32 + 16) = make_uint4(code[4], code[5], code[6], code[7]);
       }
+    } else if constexpr (kFour) {  // quads 2 p and 2 p + 1 of 4 lines
+      const int at = j & ~3, p = j & 3;
+#pragma unroll
+      for (int l = 0; l < 4; ++l) {
+        if constexpr (kPacked) {
+          *reinterpret_cast<uint32_t*>(dst + (at + l) * 16 + p * 4) = nibbles(code[2 * l]) | (nibbles(code[2 * l + 1]) << 16);
+        } else {
+          *reinterpret_cast<uint2*>(dst + (at + l) * 32 + p * 8) = make_uint2(code[2 * l], code[2 * l + 1]);
+        }
+      }
     } else {
       constexpr int kLb = kHalf ? 0 : 3 - kRC;
       const int la = (j >> 3) & ((1 << kRC) - 1);
@@ -307,11 +337,13 @@ __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(cons
   }
   if (xsum != nullptr) {
     unsigned int cs = sum_acc - 8u * 32u;  // every code carried an offset of 8
-    if ((tpr & 31) == 0) {
+    if (row_warp) {
       cs = __reduce_add_sync(0xffffffffu, cs);
-      if (!one_warp && (tid & 31) == 0) atomicAdd(&s_sum[rloc], cs);
-    } else if (rloc < rpc) {
-      atomicAdd(&s_sum[rloc], cs);
+      if (!one_warp && (tid & 31) == 0 && rloc < rpc) atomicAdd(&s_sum[rloc], cs);
+    } else {
+      cs += __shfl_xor_sync(0xffffffffu, cs, 1);
+      cs += __shfl_xor_sync(0xffffffffu, cs, 2);
+      if ((tid & 3) == 0 && rloc < rpc) atomicAdd(&s_sum[rloc], cs);
     }
     if (!one_warp) {
       __syncthreads();
@@ -328,6 +360,7 @@ cudaError_t launch_wide_t(const RotQuantArgs& a) {
   if (rows > kWideRows) rows = kWideRows;
   while (rows > 1 && (a.M + rows - 1) / rows < a.num_sms) rows /= 2;  // few rows: more CTAs, down to one row each
   const int tpb = (rows * tpr + 31) & ~31;  // whole warps: the warp-wide steps take every lane
+  rows = tpb / tpr;                         // as the kernel counts them
   auto kern = rotate_quant_wide_kernel<T, kLogB, kStep, kPacked>;
   const size_t smem = kLogB > 5 ? static_cast<size_t>(tpb) * 128 : 0;
   if (smem > 48 * 1024) {

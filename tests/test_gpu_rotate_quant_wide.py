@@ -68,7 +68,8 @@ def _values(rng, M, K, had, dt, special=True):
     (65, 128, 128, "f16", 64), (70, 384, 32, "bf16", 16), (131, 256, 64, "f16", 32), (130, 768, 256, "bf16", 8),
     (129, 512, 512, "bf16", 16), (66, 2560, 512, "f16", 4), (100, 1024, 1024, "bf16", 8), (97, 3072, 1024, "f16", 4),
     (130, 2048, 2048, "bf16", 4), (70, 6144, 2048, "f16", 1), (66, 16384, 2048, "bf16", 1), (200, 640, 1, "f16", 16),
-    (66, 4096, 16, "bf16", 2), (9, 2048, 256, "f16", 4), (50, 1024, 64, "bf16", 8)])
+    (66, 4096, 16, "bf16", 2), (9, 2048, 256, "f16", 4), (50, 1024, 64, "bf16", 8),
+    (77, 640, 128, "bf16", 16), (300, 896, 64, "f16", 16)])
 def test_a_batch_equals_the_pass_kernel_on_repeated_rows(M, K, had, dt, r):
     rng = np.random.default_rng(M + K + had)
     x = _values(rng, M, K, had, dt)
@@ -97,7 +98,8 @@ def test_a_batch_equals_the_pass_kernel_on_repeated_rows(M, K, had, dt, r):
     wide.close()
 
 
-@pytest.mark.parametrize("M,K,had", [(67, 2304, 256), (131, 1024, 1024), (70, 4096, 2048), (65, 384, 32), (33, 8192, 4096)])
+@pytest.mark.parametrize("M,K,had", [(67, 2304, 256), (131, 1024, 1024), (70, 4096, 2048), (65, 384, 32), (33, 8192, 4096),
+                                      (33, 2944, 128), (40, 10112, 64)])
 def test_f32_rows_equal_bf16_rows_of_the_same_values(M, K, had):
     rng = np.random.default_rng(K)
     xb = _values(rng, M, K, had, "bf16")
@@ -106,7 +108,7 @@ def test_f32_rows_equal_bf16_rows_of_the_same_values(M, K, had):
 
 
 @pytest.mark.parametrize("M,K,had", [(80, 1024, 64), (66, 2048, 128), (130, 4096, 2048), (1, 4096, 4096),
-                                      (66, 8192, 4096), (50, 4096, 4096)])
+                                      (66, 8192, 4096), (50, 4096, 4096), (142, 2944, 64), (70, 10112, 128), (500, 384, 128)])
 def test_step_codes_equal_the_64_channel_kernel(M, K, had):
     """A per-group table of one repeated scale runs the 64-channel kernel: the same outputs follow."""
     rng = np.random.default_rng(K + had)
