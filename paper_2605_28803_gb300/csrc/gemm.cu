@@ -81,24 +81,25 @@ TileShape token_major_shape(const GemmArgs& a, int* parts, long* estimate = null
 // token-major kernel at every shape measured (M 129-8192 and gated M 5-128, N 16-32768: 1.05 to 2.8 times); below, the
 // estimates decide.  Up to 128 tokens a layer that is not gated keeps the weight-major kernel: alone the other is faster
 // from K N = 2^21 or so, but between the small kernels of a chain it is not (the action head's step at 50 tokens: 240
-// against 221 us), as its pairs fill the SMs' shared memory and TMEM and so start late.
+// against 221 us), as its pairs fill the SMs' shared memory and TMEM and so start late.  Packed 4-bit codes go by the estimates
+// at every K, the token-major one an eighth up, as it was fitted to operand bytes (2328 x 3200 -> 1536: 19.0 us token-major
+// and 20.2 here; 400 x 2048 -> 8192 14.2 and 14.7; 1000 x 1024 -> 16384 30.2 and 24.7).
 bool take_tmem(const GemmArgs& a, int* bn, int* parts) {
   if (a.num_sms < 2 || (!a.gated && a.M <= 128)) return false;
   const long t = gemm_tmem_plan(a, bn, parts);
-  if (a.K >= 768) return true;
+  if (a.K >= 768 && a.x_bytes != 0) return true;
   int unused = 1;
   long old = 0;
   token_major_shape(a, &unused, &old);
+  if (a.x_bytes == 0) old += old / 8;
   if (a.gated && old < 6900) old = 6900;  // a gated tile's epilogue outlasts a few k-blocks
   return t < old;
 }
 
 template <int kX, typename OutT>
 cudaError_t launch_out(const GemmArgs& a) {
-  if constexpr (kX >= 1) {
-    int bn = 0, parts = 1;
-    if (take_tmem(a, &bn, &parts)) return launch_gemm_tmem(a, bn, parts);
-  }
+  int bn = 0, parts = 1;
+  if (take_tmem(a, &bn, &parts)) return launch_gemm_tmem(a, bn, parts);
   if (a.gated || a.M > 128) {
     if constexpr (kX == 2) {
       // 8-bit activation planes: single CTAs; tile width by waves x tile width

@@ -31,7 +31,11 @@
 //
 // GEMM alone, in us, token-major kernel before and this one: 816 x 2048 -> 2 x 16384 gated 60.4 and 41.1 (2660 TFLOP/s
 // of the integer product); 816 x 16384 -> 2048 38.0 and 26.9; 8192 x 2048 -> 16384 240 and 146 (3770 TFLOP/s); 3200 x
-// 16384 -> 2048 104.6 and 58.4 (3680 TFLOP/s); 8-bit codes, 816 x 2048 -> 2 x 16384 gated 79 and 61.  Bound now by the
+// 16384 -> 2048 104.6 and 58.4 (3680 TFLOP/s); 8-bit codes, 816 x 2048 -> 2 x 16384 gated 79 and 61.  Packed 4-bit codes,
+// expanded by the converters next to the weights: 777 x 4096 -> 1024 18.0 and 12.5, 5781 x 3712 -> 7392 142 and 121, 816 x
+// 2048 -> 2 x 16384 gated 72 and 57, 50 x 2048 -> 2 x 4096 gated 15.1 and 8.1; a k-block costs the converters 235 to 290 ns
+// there (the codes fetched before the wait for the TMEM stage, and the proxy fence moved up to the stores, were slower: 40
+// against 34 us at 200 x 16384 -> 2048).  Bound now by the
 // issue round of the MMA warp (about 430 cycles a k-block up to bn = 160) and the refill of the TMEM stages (about 470 at
 // 192), against 384 cycles of tensor work at bn = 192.
 #include "gemm_kernel.cuh"
@@ -93,11 +97,14 @@ __device__ __forceinline__ void tm_epi_sync() {
 // kGated: the weight tile is 128 hidden units; CTA r of the pair takes units 64 r .. 64 r + 63, gate and up rows, in
 // TMEM lanes 32 q + i (gate of unit 64 r + 16 q + i) and 32 q + 16 + i (its up row), i < 16.
 // kPlanes: operand tiles of the activations per k-block (2: the high and low nibbles of 8-bit codes).
-template <bool kGated, int kPlanes, typename OutT>
+// kPacked: the activations are packed int4 codes; the converters of a k-block expand its tokens too, into tiles as many and as
+// long in use as the weight stages in TMEM.
+template <bool kGated, int kPlanes, bool kPacked, typename OutT>
 __global__ void __launch_bounds__(kTmThreads, 1) gemm_tmem_kernel(const __grid_constant__ CUtensorMap tmap_x,
                                                                   const __grid_constant__ CUtensorMap tmap_w,
                                                                   const __grid_constant__ CUtensorMap tmap_y, TmParams p) {
   constexpr int kKb = 2 / kPlanes;  // k-blocks per ring stage
+  static_assert(!kPacked || kPlanes == 1, "packed 4-bit codes");
   extern __shared__ uint8_t dyn_smem[];
   uint8_t* const smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(dyn_smem) + 1023) & ~uintptr_t(1023));
   __shared__ __align__(8) uint64_t bar_rfull[kTmMaxStages];   // packed weights landed
@@ -119,15 +126,16 @@ __global__ void __launch_bounds__(kTmThreads, 1) gemm_tmem_kernel(const __grid_c
   const int unit0 = static_cast<int>(blockIdx.x >> 1), ustep = static_cast<int>(gridDim.x >> 1);
   const int btile = bn / 2 * kBK;               // bytes of one activation tile of this CTA
   uint8_t* const out_smem = smem;               // [half][2][kTmOut] output chunks
-  uint8_t* const ring_b = smem + kTmOutBytes;   // [S][2][bn / 2][128], 128-byte swizzled
-  uint8_t* const ring_r = ring_b + S * 2 * btile;  // [S][kKb][128][64] (gated: [S][gate, up][kKb][64][64]), 64-byte swizzled
+  uint8_t* const ring_b = smem + kTmOutBytes;   // [S (packed codes: SA)][2][bn / 2][128], 128-byte swizzled
+  uint8_t* const ring_r = ring_b + (kPacked ? SA : S) * 2 * btile;  // [S][kKb][128][64] (gated: [S][gate, up][kKb][64][64]), 64-byte swizzled
+  uint8_t* const ring_x = ring_r + S * kKb * kTmRaw;  // packed codes: [S][2][bn / 2][64]
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < S; ++s) {
-      mbar_init(smem_u32(&bar_rfull[s]), 1);
+      mbar_init(smem_u32(&bar_rfull[s]), kPacked ? 2 : 1);  // the expected bytes, of packed activations too
       mbar_init(smem_u32(&bar_rempty[s]), 2 * kTmGroups);
       for (int h = 0; h < kKb; ++h) {  // the expected bytes, the k-block's converter warps of both CTAs
-        mbar_init(smem_u32(&bar_full[s][h]), (h == 0 ? 1 : 0) + 4 * kTmGroups / kKb);
+        mbar_init(smem_u32(&bar_full[s][h]), (h == 0 && !kPacked ? 1 : 0) + 4 * kTmGroups / kKb);
         mbar_init(smem_u32(&bar_empty[s][h]), 1);
       }
     }
@@ -174,6 +182,19 @@ __global__ void __launch_bounds__(kTmThreads, 1) gemm_tmem_kernel(const __grid_c
           unit_at(u, tile, ta, tb, ka, kz);
           const int row = ta * bn + static_cast<int>(rank) * (bn / 2);
           for (int kb = ka; kb < kz; kb += kKb, ++it) {
+            if constexpr (kPacked) {  // this CTA's codes, for its own converters
+              if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_rempty[s]), ph ^ 1u))) { ok = false; break; }
+              const uint32_t bar = smem_u32(&bar_rfull[s]), dst = smem_u32(ring_x + s * btile);
+              const bool two = kb + 1 < kz;
+              if (elect_one()) {
+                mbar_arrive_expect_tx(bar, static_cast<uint32_t>((two ? 2 : 1) * (btile / 2)));
+                tma_load_2d(dst, &tmap_x, kb * (kBK / 2), row, bar);
+                if (two) tma_load_2d(dst + btile / 2, &tmap_x, (kb + 1) * (kBK / 2), row, bar);
+              }
+              __syncwarp();
+              if (++s == S) { s = 0; ph ^= 1u; }
+              continue;
+            }
             if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_empty[s][kKb - 1]), ph ^ 1u))) { ok = false; break; }
             // both CTAs' tiles complete on the leader's barrier; a unit's last stage may hold one k-block only
             const uint32_t fb = smem_u32(&bar_full[s][0]);
@@ -192,7 +213,11 @@ __global__ void __launch_bounds__(kTmThreads, 1) gemm_tmem_kernel(const __grid_c
         // before leaving, let every load land: the MMAs that read a stage release it
         for (int i = 0; i < S && i < it; ++i) {
           if (--s < 0) { s = S - 1; ph ^= 1u; }
-          ok = ok && mbar_wait(smem_u32(&bar_empty[s][kKb - 1]), ph);  // (after a time-out no MMA will release the rest)
+          if constexpr (kPacked) {
+            ok = ok && mbar_wait(smem_u32(&bar_rfull[s]), ph);
+          } else {
+            ok = ok && mbar_wait(smem_u32(&bar_empty[s][kKb - 1]), ph);  // (after a time-out no MMA will release the rest)
+          }
         }
       }
       __syncwarp();
@@ -247,7 +272,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) gemm_tmem_kernel(const __grid_c
           const uint32_t d = tmem + static_cast<uint32_t>(buf * bn);
           for (int kb = ka; kb < kz; kb += kKb) {
             const uint32_t a = tmem_a + static_cast<uint32_t>(sa * kKb * 32);
-            const uint32_t b = (desc_lo | (b0 >> 4)) + static_cast<uint32_t>(s) * b_stage;
+            const uint32_t b = (desc_lo | (b0 >> 4)) + static_cast<uint32_t>(kPacked ? sa : s) * b_stage;
 #pragma unroll
             for (int h = 0; h < kKb; ++h) {
               const bool real = h == 0 || kb + h < kz;  // a unit's last stage may hold one k-block: its release only
@@ -343,6 +368,17 @@ __global__ void __launch_bounds__(kTmThreads, 1) gemm_tmem_kernel(const __grid_c
       } else {
         tmem_st16(dst, o);
       }
+      if constexpr (kPacked) {  // this k-block's tokens: a thread per 16 bytes (32 codes) of a row
+        const uint8_t* const xs = ring_x + s * btile + half * (btile / 2);
+        uint8_t* const xd = ring_b + sa * 2 * btile + half * btile;
+#pragma unroll 1
+        for (int i = (warp & 3) * 32 + lane; i < bn * 2; i += 128) {
+          const uint4 c = *reinterpret_cast<const uint4*>(xs + i * 16);
+          const int r = i >> 2, q = (2 * i) & 6;
+          store_chunk(xd + r * 128, (q ^ (r & 7)) << 4, ((q + 1) ^ (r & 7)) << 4, c);
+        }
+        __syncwarp();
+      }
       // the store consumed every loaded value: this warp's loads of the stage have completed
       if (lane == 0) mbar_arrive(smem_u32(&bar_rempty[s]));
       const uint32_t full = smem_u32(&bar_full[s][half]);
@@ -350,6 +386,7 @@ __global__ void __launch_bounds__(kTmThreads, 1) gemm_tmem_kernel(const __grid_c
       advance();
       __syncwarp();
       tmem_st_wait();
+      if constexpr (kPacked) fence_proxy_async_smem();  // the tokens are read by the async proxy
       tc_fence_before();
       __syncwarp();
       if (lane == 0) {
@@ -573,6 +610,20 @@ cudaError_t make_tmap_weights(CUtensorMap* m, const void* base, size_t chunks, i
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+// Packed codes [rows][width bytes], read in boxes of box_rows rows of a k-block's 64 bytes, as they are.
+cudaError_t make_tmap_packed(CUtensorMap* m, const void* base, int rows, int width, int box_rows) {
+  PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
+  if (!enc) return cudaErrorNotSupported;
+  const cuuint64_t dims[2] = {static_cast<cuuint64_t>(width), static_cast<cuuint64_t>(rows)};
+  const cuuint64_t strides[1] = {static_cast<cuuint64_t>(width)};
+  const cuuint32_t box[2] = {kBK / 2, static_cast<cuuint32_t>(box_rows)};
+  const cuuint32_t estr[2] = {1, 1};
+  CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(base), dims, strides, box, estr,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 // The output [M][width] of 16-bit values, written in boxes of 64 channels x 32 tokens from 128-byte swizzled rows.
 cudaError_t make_tmap_out(CUtensorMap* m, void* base, int rows, int width) {
   PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
@@ -586,9 +637,9 @@ cudaError_t make_tmap_out(CUtensorMap* m, void* base, int rows, int width) {
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-template <bool kGated, int kPlanes, typename OutT>
+template <bool kGated, int kPlanes, bool kPacked, typename OutT>
 cudaError_t launch_tm(const GemmArgs& a, int bn, int parts) {
-  auto kern = gemm_tmem_kernel<kGated, kPlanes, OutT>;
+  auto kern = gemm_tmem_kernel<kGated, kPlanes, kPacked, OutT>;
   cudaError_t e = prepare_kernel(reinterpret_cast<const void*>(kern), kTmOutBytes + kTmSmem + 1024);
   if (e != cudaSuccess) return e;
   TmParams p;
@@ -602,9 +653,14 @@ cudaError_t launch_tm(const GemmArgs& a, int bn, int parts) {
   p.N = a.N;
   p.nkb = a.K / kBK;
   p.bn = bn;
-  p.stages = kTmSmem / (2 * (bn / 2) * kBK + (2 / kPlanes) * kTmRaw);
-  if (p.stages > kTmMaxStages) p.stages = kTmMaxStages;
+  const int btile = bn / 2 * kBK, raw = (2 / kPlanes) * kTmRaw;
   p.stages_a = (512 - 2 * bn) / (32 * (2 / kPlanes));
+  if (kPacked) {  // the expanded tokens are as deep as the weight stages, the packed codes as the packed weights
+    while ((p.stages = (kTmSmem - p.stages_a * 2 * btile) / (raw + btile)) < p.stages_a + 2) --p.stages_a;
+  } else {
+    p.stages = kTmSmem / (2 * btile + raw);
+  }
+  if (p.stages > kTmMaxStages) p.stages = kTmMaxStages;
   if (p.stages_a > p.stages - 2) p.stages_a = p.stages - 2;
   p.tiles_m = (a.M + bn - 1) / bn;
   p.tiles_n = (a.N + 255) / 256;
@@ -613,7 +669,7 @@ cudaError_t launch_tm(const GemmArgs& a, int bn, int parts) {
   p.part_cnt = a.part_cnt;
   p.kconst = (kPlanes == 2 ? 1024.0f : 64.0f) * static_cast<float>(a.K);
   CUtensorMap tx = {}, tw = {}, ty = {};
-  e = make_tmap_bytes(&tx, a.xq, a.M, kPlanes * a.K, bn / 2);
+  e = kPacked ? make_tmap_packed(&tx, a.xq, a.M, a.K / 2, bn / 2) : make_tmap_bytes(&tx, a.xq, a.M, kPlanes * a.K, bn / 2);
   if (e == cudaSuccess) e = make_tmap_weights(&tw, a.wq, static_cast<size_t>(p.tiles_n) * 2 * p.nkb, kGated ? 64 : 128, 2 / kPlanes);
   if (e == cudaSuccess) e = make_tmap_out(&ty, a.y, a.M, a.gated ? a.N / 2 : a.N);
   if (e != cudaSuccess) return e;
@@ -640,13 +696,15 @@ cudaError_t launch_tm(const GemmArgs& a, int bn, int parts) {
 // Estimated time (ns) of a launch with tiles of bn tokens in `parts` work units, fitted to GB300 measurements (M 5-8192,
 // K 128-16384, N 16-32768; over 1876 shapes within 16%, half of them within 3%): a fixed cost, more with more pairs at
 // work, with the last tile's epilogue; the first unit's k-blocks (165 ns each up to bn = 128, 172 at 160, 200 at 192; two
-// planes 250, or 1.95 bn); per further wave of pairs a unit's k-blocks and hand-over, or the epilogue where that is
+// planes 250, or 1.95 bn; packed codes 235 to 290); per further wave of pairs a unit's k-blocks and hand-over, or the epilogue where that is
 // longer; with K split, the partial's write and read-back.
 long tm_estimate(const GemmArgs& a, int bn, int parts) {
   const long pairs = a.num_sms / 2, nkb = a.K / kBK;
   const long units = static_cast<long>((a.M + bn - 1) / bn) * ((a.N + 255) / 256) * parts;
   const long waves = (units + pairs - 1) / pairs;
-  const long kb = a.x_bytes == 2 ? (bn <= 128 ? 250 : 195l * bn / 100) : bn <= 128 ? 165 : bn <= 160 ? 172 : 200;
+  const long kb = a.x_bytes == 2   ? (bn <= 128 ? 250 : 195l * bn / 100)
+                  : a.x_bytes == 0 ? (bn <= 64 ? 235 : bn <= 96 ? 264 : bn <= 128 ? 270 : bn <= 160 ? 285 : 290)
+                                   : (bn <= 128 ? 165 : bn <= 160 ? 172 : 200);
   const long work = (nkb + parts - 1) / parts * kb;
   const long split = parts > 1 ? 1500 + 7l * parts * bn : 0;
   long unit = work + (bn > 160 ? 580 : 870) + (a.gated ? 150 : 0);
@@ -655,9 +713,9 @@ long tm_estimate(const GemmArgs& a, int bn, int parts) {
   return 3000 + 28 * (units < pairs ? units : pairs) + 8l * bn + (a.gated ? 200 : 0) + work + split + (waves - 1) * (unit + split);
 }
 
-template <int kPlanes, typename OutT>
+template <int kPlanes, bool kPacked, typename OutT>
 cudaError_t launch_tm_g(const GemmArgs& a, int bn, int parts) {
-  return a.gated ? launch_tm<true, kPlanes, OutT>(a, bn, parts) : launch_tm<false, kPlanes, OutT>(a, bn, parts);
+  return a.gated ? launch_tm<true, kPlanes, kPacked, OutT>(a, bn, parts) : launch_tm<false, kPlanes, kPacked, OutT>(a, bn, parts);
 }
 
 }  // namespace
@@ -692,8 +750,11 @@ long gemm_tmem_plan(const GemmArgs& a, int* bn, int* parts) {
 }
 
 cudaError_t launch_gemm_tmem(const GemmArgs& a, int bn, int parts) {
-  if (a.x_bytes == 2) return a.ydt == 0 ? launch_tm_g<2, __half>(a, bn, parts) : launch_tm_g<2, __nv_bfloat16>(a, bn, parts);
-  return a.ydt == 0 ? launch_tm_g<1, __half>(a, bn, parts) : launch_tm_g<1, __nv_bfloat16>(a, bn, parts);
+  if (a.x_bytes == 2)
+    return a.ydt == 0 ? launch_tm_g<2, false, __half>(a, bn, parts) : launch_tm_g<2, false, __nv_bfloat16>(a, bn, parts);
+  if (a.x_bytes == 0)
+    return a.ydt == 0 ? launch_tm_g<1, true, __half>(a, bn, parts) : launch_tm_g<1, true, __nv_bfloat16>(a, bn, parts);
+  return a.ydt == 0 ? launch_tm_g<1, false, __half>(a, bn, parts) : launch_tm_g<1, false, __nv_bfloat16>(a, bn, parts);
 }
 
 cudaError_t read_and_clear_error_word_tmem(unsigned int* out, cudaStream_t stream) {

@@ -1,8 +1,9 @@
 """GPU parity of the GEMM on CTA pairs with the expanded weights in TMEM (csrc/gemm_tmem.cu; Sec. 4.2, Eq. 7).
 
 qvla_w4a4_linear's GEMM takes it for batches of more than 128 tokens and for gated layers from 5 (below K = 768 where it is
-estimated faster); qvla_gemm_w4a4 on the same codes, packed, runs the token-major kernel.  Every accumulation is exact and the epilogue is the same operations, so the outputs must be the
-same bits.  Shapes sit at the edges of its tiles: one k-block and odd counts of them (the last ring stage holds one), token
+estimated faster); qvla_gemm_w4a4 takes packed codes there where it is estimated faster, else to the token-major kernel, and
+expands them in its converters.  Every accumulation is exact and the epilogue is the same operations, so the outputs must be
+the same bits, also of slices of a few tokens, which run the weight-major kernel and the GEMV.  Shapes sit at the edges of its tiles: one k-block and odd counts of them (the last ring stage holds one), token
 counts around the tile widths, weight rows past 64-, 128- and 256-row boundaries, tiles in several waves, K split into work
 units, and gated layers from a few tokens.  With 8-bit codes the accumulators must be the oracle's integers."""
 
@@ -68,6 +69,35 @@ def test_gated_equals_the_token_major_kernel(M, K, H, dt):
     x = torch.from_numpy(rng.standard_normal((M, K), dtype=np.float32)).to(_T[dt]).to(G.DEV)
     y, ref = _both(layer, x, M, dt)
     assert torch.equal(y, ref)
+    layer.close()
+
+
+@pytest.mark.parametrize("M,K,N,gated,dt", [
+    (129, 768, 16, False, "f16"), (150, 896, 512, False, "bf16"), (777, 4096, 1024, False, "f16"), (200, 16384, 2048, False, "bf16"),
+    (500, 384, 528, False, "f16"), (2500, 1152, 2560, False, "bf16"), (4001, 1024, 4112, False, "f16"), (10, 1024, 2048, True, "bf16"),
+    (50, 2176, 384, True, "f16"), (193, 1152, 1024, True, "bf16")])
+def test_packed_codes_equal_slices_of_few_tokens(M, K, N, gated, dt):
+    """Packed codes: the weight-major kernel (up to 128 tokens) and, for gated layers, the GEMV (4 tokens) on slices."""
+    rng = np.random.default_rng(M + K + N)
+    layer, _ = _layer(rng, N, K, 128, dt, gated)
+    xq = torch.from_numpy(rng.integers(0, 256, (M, K // 2), dtype=np.uint8)).to(G.DEV)
+    xq = torch.where((xq & 15) == 8, xq ^ 8, xq)  # codes -7 .. 7
+    xq = torch.where((xq >> 4) == 8, xq ^ 0x80, xq)
+    nib = torch.stack((xq & 15, xq >> 4), 2).to(torch.int32)
+    xsum = ((nib ^ 8) - 8).sum((1, 2), dtype=torch.int32)
+    xs = torch.from_numpy(rng.uniform(0.5, 1.5, M).astype(np.float32) / 64).to(G.DEV)
+    y = torch.full((M, N), float("nan"), dtype=_T[dt], device=G.DEV)
+    acc = torch.full((M, 2 * N if gated else N), -1, dtype=torch.int32, device=G.DEV)
+    Q.qvla_gemm_w4a4(layer, xq, xs, xsum, M, y, acc, G.stream())
+    rows = 4 if gated else 128
+    for i in range(0, M, rows):
+        m = min(rows, M - i)
+        part = torch.empty(m, N, dtype=_T[dt], device=G.DEV)
+        pacc = torch.empty(m, acc.shape[1], dtype=torch.int32, device=G.DEV)
+        Q.qvla_gemm_w4a4(layer, xq[i : i + m].clone(), xs[i : i + m].clone(), xsum[i : i + m].clone(), m, part, pacc, G.stream())
+        assert torch.equal(acc[i : i + m], pacc)
+        assert torch.equal(y[i : i + m], part)
+    Q.qvla_check_device(G.stream())
     layer.close()
 
 
