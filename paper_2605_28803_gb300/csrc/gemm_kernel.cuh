@@ -425,6 +425,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w4a4_kernel(const __grid_con
   __shared__ __align__(16) float s_ws[kSwap ? 1 : kBN];
   __shared__ __align__(16) float s_wc[kSwap ? 1 : kBN];
   __shared__ __align__(16) float s_bs[kSwap ? 1 : kBN];
+  __shared__ __align__(16) float s_gc[2][kGroup ? kBN : 2];  // grouped: the columns' corrections, of two groups in turn
 
   const int warp = warp_index();
   const int lane = threadIdx.x & 31;
@@ -876,23 +877,36 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w4a4_kernel(const __grid_con
         const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(warp * 32) << 16);
         const uint32_t run = lane_base + static_cast<uint32_t>(2 * kBN);  // the running sum's columns
         const int ra = ta * kBM + et;  // this thread's MMA-A row
-        bool ok = true;
+        const bool rok = ra < (kSwap ? p.N : p.M);
+        // A group's parameters, fetched one group ahead: its scale, the correction of this thread's row, and of column et
+        // (every thread needs those of all columns: they go through shared memory.  Loaded where they are used, one
+        // at a time and all lanes alike, they took most of a group's 2.1 us)
+        const int* const xg = p.xgsum + static_cast<size_t>(kSwap ? min(tb * kBN + et, p.M - 1) : (rok ? ra : 0)) * G;
+        const float* const wg = p.wgcorr + static_cast<size_t>(kSwap ? (rok ? ra : 0) : min(tb * kBN + et, p.N - 1)) * G;
+        float f_dg = __ldg(p.gscale + g0), f_w = __ldg(wg + g0);
+        int f_x = __ldg(xg + g0);
         for (int g = g0; g < g1; ++g, ++gi) {
           const int buf = gi & 1;
+          // the fixed part of this row's correction: 8 x its code sum over the group + 64 x size
+          const float xcorr = 8.0f * static_cast<float>(f_x);
+          const float rcorr = (kSwap ? f_w : xcorr) + gconst, dg = f_dg;
+          if (et < kBN) s_gc[buf][et] = kSwap ? xcorr : f_w;
+          if (g + 1 < g1) {
+            f_dg = __ldg(p.gscale + g + 1);
+            f_w = __ldg(wg + g + 1);
+            f_x = __ldg(xg + g + 1);
+          }
+          epi_sync();  // the column corrections are there, and those of two groups ago no longer read
+          if (s_epi_abort) break;
           if (!mbar_wait(smem_u32(&bar_tfull[buf]), static_cast<uint32_t>(gi >> 1) & 1u)) {
-            s_epi_abort = 1;
-            ok = false;
-            break;
+            s_epi_abort = 1;  // every thread leaves after the next barrier
+            continue;
           }
           tc_fence_after();
           const uint32_t part = lane_base + static_cast<uint32_t>(buf * kBN);
-          const float dg = __ldg(p.gscale + g);
           const bool first = g == g0, last = g == g1 - 1;
-          // the fixed part of this row's correction: 8 x its code sum over the group + 64 x size
-          const bool rok = ra < (kSwap ? p.N : p.M);
-          const int rc = rok ? ra : 0;
-          const float rcorr = kSwap ? __ldg(p.wgcorr + static_cast<size_t>(rc) * G + g) + gconst
-                                    : 8.0f * static_cast<float>(__ldg(p.xgsum + static_cast<size_t>(rc) * G + g)) + gconst;
+          const float2 rc2 = make_float2(rcorr, rcorr), dg2 = make_float2(dg, dg);
+          const float2 unit2 = make_float2(262144.0f, 262144.0f), neg2 = make_float2(-1.0f, -1.0f);
 #pragma unroll 1
           for (int c0 = 0; c0 < kBN; c0 += kChunk) {
             uint32_t r[32], R[32];
@@ -907,13 +921,14 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w4a4_kernel(const __grid_con
             tmem_ld_wait();
             const int col0 = tb * kBN + c0;  // first column (token when swapped, weight row else)
 #pragma unroll
-            for (int i = 0; i < kChunk; ++i) {
-              const int col = min(col0 + i, (kSwap ? p.M : p.N) - 1);
-              const float ccorr = kSwap ? 8.0f * static_cast<float>(__ldg(p.xgsum + static_cast<size_t>(col) * G + g))
-                                        : __ldg(p.wgcorr + static_cast<size_t>(col) * G + g);
+            for (int i = 0; i < kChunk; i += 2) {
+              const float2 cc = __fadd2_rn(rc2, *reinterpret_cast<const float2*>(&s_gc[buf][c0 + i]));
               // exact: the group's integer accumulator, below 2^24
-              const float acc = fmaf(__uint_as_float(r[i]), 262144.0f, -(rcorr + ccorr));
-              R[i] = __float_as_uint(fmaf(dg, acc, first ? 0.0f : __uint_as_float(R[i])));
+              const float2 acc = __ffma2_rn(make_float2(__uint_as_float(r[i]), __uint_as_float(r[i + 1])), unit2, __fmul2_rn(cc, neg2));
+              const float2 sum = first ? make_float2(0.0f, 0.0f) : make_float2(__uint_as_float(R[i]), __uint_as_float(R[i + 1]));
+              const float2 y2 = __ffma2_rn(dg2, acc, sum);
+              R[i] = __float_as_uint(y2.x);
+              R[i + 1] = __float_as_uint(y2.y);
             }
             if (!last) {
               if constexpr (kChunk == 32) {
@@ -953,7 +968,6 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w4a4_kernel(const __grid_con
           tc_fence_before();
           mbar_arrive(smem_u32(&bar_tempty[buf]));
         }
-        if (!ok) continue;
       }
     } else
     for (int u = QVLA_UNIT0; u < nunits; u += QVLA_NUNITS, ++tile_iter) {
