@@ -14,10 +14,11 @@ cudaError_t launch_rotate_quant_a8_bf16(const RotQuantArgs& a);
 cudaError_t launch_rotate_quant_a8_f32(const RotQuantArgs& a);
 
 // The kernel with 32 channels per thread (rotate_quant_wide.cuh): 4-bit codes with one scale per row (per token or per
-// step).  K is a multiple of 128 and of the block, which is all that its groups of threads need.
+// step), or per step and group of up to 1024 channels, whose 32 threads sum their codes within a warp.  K is a multiple of
+// 128 and of the block, which is all that its groups of threads need.
 static bool rotate_quant_wide_takes(const RotQuantArgs& a) {
-  return (a.mode == 0 || a.mode == 1) && (a.out_mode == 0 || a.out_mode == 1) && a.gshift >= 30 && a.xgsum == nullptr &&
-         a.log_b >= 0 && a.log_b <= 12;
+  const bool rows = a.gshift >= 30 && a.xgsum == nullptr, groups = a.mode == 1 && a.gshift <= 10;
+  return (a.mode == 0 || a.mode == 1) && (a.out_mode == 0 || a.out_mode == 1) && (rows || groups) && a.log_b >= 0 && a.log_b <= 12;
 }
 
 bool rotate_quant_supported(int log_b) { return log_b >= 0 && log_b <= 12; }

@@ -1,7 +1,7 @@
 // Fused online rotation + symmetric 4-bit activation quantisation (Sec. 4.1 Eq. 3-5, Sec. 4.2 Eq. 5-6) for batches of rows:
 // 32 channels per thread, codes by packed E4M3 conversion.
 //
-// It does what rotate_quant.cuh's kernel does for 4-bit codes and one scale per row, bit for bit, with fewer instructions
+// It does what rotate_quant.cuh's kernel does for 4-bit codes, bit for bit, with fewer instructions
 // per channel and twice the warps in flight:
 //   * a thread holds 32 channels instead of 64: 64 registers, 32 warps per SM;
 //   * the butterflies run in three phases, index bits 0-4 on 32 consecutive channels, 5-7 (5-6 among 4 threads for blocks of
@@ -18,7 +18,8 @@
 // Measured back to back in a graph, 64-channel kernel before and this one, us: 816 x 2048 bf16 5.9 and 4.8; 816 x 16384
 // 23.0 and 18.0; 3200 x 16384 f16 72.0 and 58.4 (2.7 TB/s of x and codes); 8192 x 2048 22.7 and 19.3; 201 x 2304 with
 // blocks of 256 3.9 and 2.8; f32 777 x 4096 9.9 and 9.7; blocks of 128: 3325 x 10112 47.3 and 32.0, 7761 x 2688 29.3 and 20.6,
-// 8192 x 384 8.6 and 5.2.  About 21 instructions a channel at 55% of the issue slots; neither
+// 8192 x 384 8.6 and 5.2; with a scale per 128-channel group the linear 50 x 1024 -> 4096 8.0 and 7.0, 5954 x 14080 -> 288
+// 233 and 223.  About 21 instructions a channel at 55% of the issue slots; neither
 // the transposes, the butterflies nor the conversions alone bound it (leaving one of them out saves 6 to 16%).  Staying
 // CTAs fed by TMA one group ahead were slower (73 us at 3200 x 16384): with an extra barrier a group, two CTAs an SM overlap
 // less than fresh ones.  A few rows are spread one to a CTA: 50 x 1024 2.1 us against 2.8 with eight rows a CTA; with blocks
@@ -87,8 +88,9 @@ template <typename T, int kLogB, bool kStep, bool kPacked>
 __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(const T* __restrict__ x, int M, int K, float inv_sqrt_b,
                                                                             const float* __restrict__ step_scale,
                                                                             uint8_t* __restrict__ xq, float* __restrict__ xscale,
-                                                                            int32_t* __restrict__ xsum, int32_t* __restrict__ zero,
-                                                                            int zero_n) {
+                                                                            int32_t* __restrict__ xsum, int gshift,
+                                                                            int32_t* __restrict__ xgsum,
+                                                                            int32_t* __restrict__ zero, int zero_n) {
   constexpr int kA = kLogB < 5 ? kLogB : 5;                        // index bits of the first phase
   constexpr int kRB = kLogB <= 5 ? 0 : kLogB < 8 ? kLogB - 5 : 3;  // of the second: 5 .. 5 + kRB - 1
   constexpr int kRC = kLogB <= 8 ? 0 : kLogB - 8;                  // of the third: 8 .. 8 + kRC - 1
@@ -213,7 +215,8 @@ __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(cons
   // ---- scale ----
   float delta;
   if constexpr (kStep) {
-    delta = __ldg(step_scale);
+    // (a scale group holds whole Hadamard blocks of at most 32 threads: this thread's channels stay in one)
+    delta = __ldg(step_scale + (gshift >= 30 ? 0 : (j * 32) >> gshift));
   } else {
     float w = 0.0f;
 #pragma unroll
@@ -335,6 +338,12 @@ __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(cons
       }
     }
   }
+  if (xgsum != nullptr) {  // the code sum of each scale group of the row (at most 32 consecutive lanes)
+    int gs = static_cast<int>(sum_acc) - 8 * 32;
+    const int tg = 1 << (gshift - 5);
+    for (int o = tg >> 1; o > 0; o >>= 1) gs += __shfl_xor_sync(0xffffffffu, gs, o);
+    if (active && (j & (tg - 1)) == 0) xgsum[static_cast<size_t>(m) * (K >> gshift) + ((j * 32) >> gshift)] = gs;
+  }
   if (xsum != nullptr) {
     unsigned int cs = sum_acc - 8u * 32u;  // every code carried an offset of 8
     if (row_warp) {
@@ -387,7 +396,7 @@ cudaError_t launch_wide_t(const RotQuantArgs& a) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   cudaError_t e = cudaLaunchKernelEx(&cfg, kern, reinterpret_cast<const T*>(a.x), a.M, a.K, a.inv_sqrt_b, a.step_scale, a.xq,
-                                     a.xscale, a.xsum, a.zero, a.zero_n);
+                                     a.xscale, a.xsum, a.gshift, a.xgsum, a.zero, a.zero_n);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }

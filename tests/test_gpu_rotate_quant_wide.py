@@ -4,8 +4,9 @@ Sec. 4.2 Eq. 5-6).
 It takes 4-bit codes with one scale per row, but for a few long rows, which the pass kernel keeps (at most 48 rows of more
 than 4096 channels; its codes, scales and sums are pinned elsewhere).  A row repeated r times side by side has the same
 rotated values, the same maximum and r times the code sum, so the pass kernel on repeated rows pins this one at every
-width.  A per-group table of equal scales runs the 64-channel kernel, which pins the per-step codes, blocks of 4096
-included.  Blocks at every phase count and group size, row widths that are not a power of two of threads, ragged rows per
+width.  A per-group table of equal scales takes the 64-channel kernel for groups of 2048 and 4096 channels, which pins the
+per-step codes of such blocks, and this kernel for smaller groups, whose codes and sums equal those of the groups taken as rows
+of their own.  Blocks at every phase count and group size, row widths that are not a power of two of threads, ragged rows per
 CTA, per token and per step with clamping, exact ties, zero rows, huge, tiny, infinite and NaN values."""
 
 import numpy as np
@@ -110,7 +111,7 @@ def test_f32_rows_equal_bf16_rows_of_the_same_values(M, K, had):
 @pytest.mark.parametrize("M,K,had", [(80, 1024, 64), (66, 2048, 128), (130, 4096, 2048), (1, 4096, 4096),
                                       (66, 8192, 4096), (50, 4096, 4096), (142, 2944, 64), (70, 10112, 128), (500, 384, 128)])
 def test_step_codes_equal_the_64_channel_kernel(M, K, had):
-    """A per-group table of one repeated scale runs the 64-channel kernel: the same outputs follow."""
+    """A per-group table of one repeated scale runs the 64-channel kernel from groups of 2048: the same outputs follow."""
     rng = np.random.default_rng(K + had)
     x = _values(rng, M, K, had, "f16", special=False)
     wq = rng.integers(0, 256, (32, K // 2), dtype=np.uint8)
@@ -130,3 +131,32 @@ def test_step_codes_equal_the_64_channel_kernel(M, K, had):
         out.append(work[: M * K].cpu())
         layer.close()
     assert torch.equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("M,K,had,dt", [(50, 1024, 64, "f16"), (142, 2944, 128, "bf16"), (700, 384, 1, "f16"), (33, 2560, 512, "bf16"),
+                                         (65, 3072, 1024, "f16"), (9, 512, 256, "bf16"), (3000, 256, 32, "f16")])
+def test_group_codes_equal_the_groups_as_rows(M, K, had, dt):
+    rng = np.random.default_rng(M + K)
+    x = _values(rng, M, K, had, dt, special=False)
+    group = max(128, had)
+    n = K // group
+    table = rng.uniform(0.05, 0.6, n).astype(np.float32)
+    layer = Q.qvla_layer_create(16, K, had, Q.DTYPE_CODES[dt], Q.F16, np.zeros((16, K // 2), np.uint8), np.ones(16, np.float32), None)
+    Q.qvla_set_step_group_scales(layer, table[None, :])
+    nb = Q.qvla_linear_workspace_bytes(layer, M)
+    work = torch.full((nb,), 0x3C, dtype=torch.uint8, device=G.DEV)
+    y = torch.empty(M, 16, dtype=torch.float16, device=G.DEV)
+    Q.qvla_w4a4_linear(layer, x, M, 0, y, work, nb, G.stream())
+    Q.qvla_check_device(G.stream())
+    r256 = lambda v: (v + 255) // 256 * 256  # noqa: E731
+    codes = work[: M * K].view(M, n, group).cpu()
+    o = r256(M * K) + 2 * r256(4 * M)
+    gsum = work[o : o + 4 * M * n].view(torch.int32).view(M, n).cpu()
+    part = Q.qvla_layer_create(16, group, had, Q.DTYPE_CODES[dt], Q.F16, np.zeros((16, group // 2), np.uint8), np.ones(16, np.float32),
+                               None)
+    Q.qvla_set_step_scales(part, table)
+    for g in range(n):
+        ob, _, xsum = _quantise(part, x[:, g * group : (g + 1) * group], g)
+        assert torch.equal(codes[:, g], ob) and torch.equal(gsum[:, g], xsum)
+    part.close()
+    layer.close()
