@@ -491,7 +491,7 @@ cudaError_t launch_t(const RotQuantArgs& a) {
   if (grid == 0) return cudaSuccess;
   const size_t smem = (kLogB > ((kEpt == 128) ? 7 : 6)) ? static_cast<size_t>(tpb) * kEpt * sizeof(float) : 0;
   auto kern = rotate_quant_kernel<T, kLogB, kEpt, kStep, kA8>;
-  if (smem > 48 * 1024) {
+  if (smem > 40 * 1024) {  // (48 KB without it, the kernel's own few words included: K = 12288 needs it)
     // raise the kernel's limit once per device to the most any K asks of it (one kernel serves
     // several K, so several sizes: at most 256 threads x 128 float32 = 128 KB)
     constexpr int kMaxSmem = 128 * 1024;

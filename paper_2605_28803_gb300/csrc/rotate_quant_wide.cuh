@@ -372,7 +372,7 @@ cudaError_t launch_wide_t(const RotQuantArgs& a) {
   rows = tpb / tpr;                         // as the kernel counts them
   auto kern = rotate_quant_wide_kernel<T, kLogB, kStep, kPacked>;
   const size_t smem = kLogB > 5 ? static_cast<size_t>(tpb) * 128 : 0;
-  if (smem > 48 * 1024) {
+  if (smem > 40 * 1024) {  // (48 KB without it, the kernel's own few words included)
     constexpr int kMaxSmem = kWideThreads * 128;  // raised once per device to the most any K asks of it
     static std::atomic<unsigned long long> raised{0};
     int dev = 0;

@@ -29,7 +29,8 @@ def _rotate(layer, x, out):
 
 
 @pytest.mark.parametrize("dt", ["f16", "bf16", "f32"])
-@pytest.mark.parametrize("M,K,block", [(2048, 1024, 64), (2049, 1024, 16), (1153, 2944, 32), (129, 16384, 64), (1025, 2176, 64)])
+@pytest.mark.parametrize("M,K,block", [(2048, 1024, 64), (2049, 1024, 16), (1153, 2944, 32), (129, 16384, 64), (1025, 2176, 64),
+                                       (171, 12288, 32)])
 def test_large_batches_equal_slices(dt, M, K, block):
     t = {"f16": torch.float16, "bf16": torch.bfloat16, "f32": torch.float32}[dt]
     layer = _layer(K, block, dt)

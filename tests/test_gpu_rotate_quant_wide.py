@@ -100,7 +100,7 @@ def test_a_batch_equals_the_pass_kernel_on_repeated_rows(M, K, had, dt, r):
 
 
 @pytest.mark.parametrize("M,K,had", [(67, 2304, 256), (131, 1024, 1024), (70, 4096, 2048), (65, 384, 32), (33, 8192, 4096),
-                                      (33, 2944, 128), (40, 10112, 64)])
+                                      (33, 2944, 128), (40, 10112, 64), (50, 12288, 4096)])
 def test_f32_rows_equal_bf16_rows_of_the_same_values(M, K, had):
     rng = np.random.default_rng(K)
     xb = _values(rng, M, K, had, "bf16")
@@ -160,3 +160,14 @@ def test_group_codes_equal_the_groups_as_rows(M, K, had, dt):
         assert torch.equal(codes[:, g], ob) and torch.equal(gsum[:, g], xsum)
     part.close()
     layer.close()
+
+
+@pytest.mark.parametrize("K", range(128, 16385, 128))
+def test_every_row_width_runs(K):
+    """Every K, with many rows a CTA and one: the shared memory and thread counts of each width are accepted, and a
+    row's code sum is that of its codes."""
+    x = torch.randn(153 if K % 256 else 80, K, device=G.DEV, dtype=torch.float16)
+    xq, _, xsum = _packed(x, 64)
+    codes = _unpack(xq).to(torch.int32) - 8
+    assert torch.equal(codes.sum(1, dtype=torch.int32), xsum)
+    assert int(codes.abs().max()) == 7
