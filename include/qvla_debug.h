@@ -29,9 +29,11 @@ extern "C" {
  * again. */
 qvla_status qvla_debug_set_hooks(unsigned long long wait_limit_ns, int hold_gemm_loads);
 
-/* The launch plan that qvla_w4a4_linear's GEMM (Sec. 4.2, Eq. 7) takes for M > 128 tokens of an
- * M x K -> N layer on a device of num_sms SMs: the host-side choice of tile shape and split of K,
- * computed without touching a device.
+/* The token-major GEMM's estimate (Sec. 4.2, Eq. 7) for M > 128 tokens of an M x K -> N layer on a
+ * device of num_sms SMs: the tile shape and split of K with the least estimated time, computed
+ * without touching a device.  The dispatch weighs it against the CTA-pair kernel with the weights in
+ * TMEM, which takes qvla_w4a4_linear's GEMM from K = 768 on and plans its own tiles and split; below,
+ * and for packed codes, the token-major kernel runs the shape in whole tiles where it is faster.
  *   N          the layer's weight rows (2H for a gated layer)
  *   gated      nonzero: a gated gate/up layer (qvla_layer_create_gated)
  *   split_room nonzero: the workspace has the room qvla_linear_workspace_bytes counts for the

@@ -24,11 +24,11 @@ cudaError_t launch_grouped(const GemmArgs& a) {
 // (2000 + 344 / k-block) and 2000 + waves x (2500 + 560 / k-block); CTA pairs (256 tokens over two
 // SMs, half the weight rows staged per SM) 3900 + waves x (1000 + 351 / k-block) and 3800 + waves
 // x (2900 + 375 / k-block).  A pair wave holds half as many tiles, each of twice the tokens.
-// A non-gated layer whose tiles leave SMs (or pairs) idle may split each tile's k-blocks into 2
-// or 4 work units of at least 16 k-blocks (their partials in the caller's workspace, the tile's
-// last unit finishing it): a wave of units then costs per_tile + split + k-blocks per unit x
+// A non-gated layer whose tiles leave SMs (or pairs) idle is estimated with each tile's k-blocks in 2
+// or 4 work units of at least 16 k-blocks: a wave of units then costs per_tile + split + k-blocks per unit x
 // per_kb, with split fitted on 816 x 16384 -> 2048: 4900 ns for single CTAs (128-wide tiles in 4
-// parts, 56.0 us against 53.9 whole) and 14500 for pairs (256-wide tiles in 2 parts, 45.2 us).
+// parts, 56.0 us against 53.9 whole) and 14500 for pairs (256-wide tiles in 2 parts, 45.2 us).  The kernel runs whole
+// tiles: launches of 16 k-blocks a unit are the TMEM kernel's (gemm_tmem.cu), with its own plan.
 enum class TileShape { kSingle128, kSingle256, kPair128, kPair256 };
 
 TileShape token_major_shape(const GemmArgs& a, int* parts, long* estimate = nullptr) {
@@ -110,19 +110,18 @@ cudaError_t launch_out(const GemmArgs& a) {
       if (w128 * 128 < w256 * 256) return launch_cfg<128, false, false, kX, OutT>(a);
       return launch_cfg<256, false, false, kX, OutT>(a);
     } else {
-      // gated layers always take 256-wide tiles: a tile's gate and up rows meet in one epilogue
-      GemmArgs b = a;
-      switch (token_major_shape(a, &b.parts)) {
-        case TileShape::kPair256:
-          return b.gated ? launch_cfg<256, false, true, kX, OutT, false, true>(b)
-                         : launch_cfg<256, false, false, kX, OutT, false, true>(b);
-        case TileShape::kPair128:
-          return launch_cfg<128, false, false, kX, OutT, false, true>(b);
-        case TileShape::kSingle128:
-          return launch_cfg<128, false, false, kX, OutT>(b);
-        default:
-          return b.gated ? launch_cfg<256, false, true, kX, OutT>(b) : launch_cfg<256, false, false, kX, OutT>(b);
+      // gated layers always take 256-wide tiles: a tile's gate and up rows meet in one epilogue.  Whole tiles: operand bytes
+      // come here below K = 768 only, where neither pairs nor a split are planned, and packed codes bring no workspace.
+      int whole = 1;
+      const TileShape shape = token_major_shape(a, &whole);
+      if constexpr (kX == 0) {
+        if (shape == TileShape::kPair256)
+          return a.gated ? launch_cfg<256, false, true, kX, OutT, false, true>(a)
+                         : launch_cfg<256, false, false, kX, OutT, false, true>(a);
+        if (shape == TileShape::kPair128) return launch_cfg<128, false, false, kX, OutT, false, true>(a);
       }
+      if (shape == TileShape::kSingle128) return launch_cfg<128, false, false, kX, OutT>(a);
+      return a.gated ? launch_cfg<256, false, true, kX, OutT>(a) : launch_cfg<256, false, false, kX, OutT>(a);
     }
   }
   const int mpad = (a.M + 15) / 16 * 16;

@@ -88,11 +88,10 @@ struct GemmArgs {
   int xdt = 0;
   int log_b = 0;
   float inv_sqrt_b = 1.0f;
-  // token-major tiles of a non-gated layer may split their k-blocks into `parts` work units
-  // when the tiles leave SMs idle: the units' FP32 partials go to part_ws (part_ws_floats
-  // floats) and part_cnt (part_cnt_n ints, zero at launch; the GEMM leaves them zero) counts
-  // each tile's finished units.  Null: no split.  `parts` is set by the tile-shape choice.
-  int parts = 1;
+  // the tiles of a non-gated layer may split their k-blocks into work units when they leave SMs
+  // idle (gemm_tmem.cu): the units' FP32 partials go to part_ws (part_ws_floats floats) and
+  // part_cnt (part_cnt_n ints, zero at launch; the GEMM leaves them zero) counts each tile's
+  // finished units.  Null: no split.
   float* part_ws = nullptr;
   size_t part_ws_floats = 0;
   int* part_cnt = nullptr;
@@ -101,10 +100,9 @@ struct GemmArgs {
   cudaStream_t stream;
 };
 cudaError_t launch_gemm_w4a4(const GemmArgs& a);
-// The token-major launch plan of launch_gemm_w4a4 for int4 operand-byte activations and M > 128
-// (host logic only; a's device pointers are not read): the tile shape (0 single CTAs 128 x 128,
-// 1 single CTAs 128 x 256, 2 CTA pairs 256 x 128, 3 CTA pairs 256 x 256) and *parts, the work
-// units per tile (1 = whole tiles).
+// The token-major kernel's estimate for int4 activations and M > 128 (host logic only; a's device pointers are not read): the
+// tile shape with the least estimated time (0 single CTAs 128 x 128, 1 single CTAs 128 x 256, 2 CTA pairs 256 x 128, 3 CTA
+// pairs 256 x 256) and *parts, the work units per tile it is estimated with.  The dispatch weighs it against gemm_tmem_plan.
 int token_major_plan(const GemmArgs& a, int* parts);
 
 // The GEMM on CTA pairs with the expanded weights in TMEM (gemm_tmem.cu): operand-byte activations (x_bytes 1 or 2), one
