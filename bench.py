@@ -259,7 +259,7 @@ class ClockSampler:
 def gemm_source_hash():
     """sha256 over the GEMM kernel's sources (the kernel template and its dispatch)."""
     h = hashlib.sha256()
-    for f in ("gemm_kernel.cuh", "gemm.cu", "ptx.cuh"):
+    for f in ("gemm_tmem.cu", "gemm_kernel.cuh", "gemm.cu", "ptx.cuh"):
         h.update(open(os.path.join(ROOT, "paper_2605_28803_gb300", "csrc", f), "rb").read())
     return h.hexdigest()
 
