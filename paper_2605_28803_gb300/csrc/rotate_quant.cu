@@ -29,19 +29,19 @@ cudaError_t launch_rotate_quant(const RotQuantArgs& a) {
     const cudaError_t e = launch_rotate_quant_pass(a, &launched);
     if (e != cudaSuccess || launched) return e;
   }
+  if (a.out_mode >= 2) {  // 8-bit codes, one scale per row
+    switch (a.xdt) {
+      case 0: return launch_rotate_quant_a8_f16(a);
+      case 1: return launch_rotate_quant_a8_bf16(a);
+      case 2: return launch_rotate_quant_a8_f32(a);
+      default: return cudaErrorInvalidValue;
+    }
+  }
   if (rotate_quant_wide_takes(a)) {
     switch (a.xdt) {
       case 0: return launch_rotate_quant_wide_f16(a);
       case 1: return launch_rotate_quant_wide_bf16(a);
       case 2: return launch_rotate_quant_wide_f32(a);
-      default: return cudaErrorInvalidValue;
-    }
-  }
-  if (a.out_mode >= 2) {
-    switch (a.xdt) {
-      case 0: return launch_rotate_quant_a8_f16(a);
-      case 1: return launch_rotate_quant_a8_bf16(a);
-      case 2: return launch_rotate_quant_a8_f32(a);
       default: return cudaErrorInvalidValue;
     }
   }

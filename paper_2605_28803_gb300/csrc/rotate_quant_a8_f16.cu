@@ -1,7 +1,8 @@
-// Rotate + quantise kernels with 8-bit codes for f16 activations (the template lives in
-// rotate_quant.cuh).
-#include "rotate_quant.cuh"
+// Rotate + quantise kernels with 8-bit codes for f16 activations (the template lives in rotate_quant_wide.cuh).
+#include "rotate_quant_wide.cuh"
 
 namespace qvla {
-cudaError_t launch_rotate_quant_a8_f16(const RotQuantArgs& a) { return rq::launch_dtype<__half, true>(a); }
+cudaError_t launch_rotate_quant_a8_f16(const RotQuantArgs& a) {
+  return a.out_mode == 2 ? rq::launch_wide<__half, 2>(a) : rq::launch_wide<__half, 3>(a);
+}
 }  // namespace qvla

@@ -1,7 +1,7 @@
 // Fused online rotation + symmetric 4-bit activation quantisation (Sec. 4.1 Eq. 3-5, Sec. 4.2 Eq. 5-6) for batches of rows:
-// 32 channels per thread, codes by packed E4M3 conversion.
+// 32 channels per thread, 4-bit codes by packed E4M3 conversion, 8-bit codes by magic-number rounding.
 //
-// It does what rotate_quant.cuh's kernel does for 4-bit codes, bit for bit, with fewer instructions
+// It does what rotate_quant.cuh's kernel does, bit for bit, with fewer instructions
 // per channel and twice the warps in flight:
 //   * a thread holds 32 channels instead of 64: 64 registers, 32 warps per SM;
 //   * the butterflies run in three phases, index bits 0-4 on 32 consecutive channels, 5-7 (5-6 among 4 threads for blocks of
@@ -19,7 +19,7 @@
 // 23.0 and 18.0; 3200 x 16384 f16 72.0 and 58.4 (2.7 TB/s of x and codes); 8192 x 2048 22.7 and 19.3; 201 x 2304 with
 // blocks of 256 3.9 and 2.8; f32 777 x 4096 9.9 and 9.7; blocks of 128: 3325 x 10112 47.3 and 32.0, 7761 x 2688 29.3 and 20.6,
 // 8192 x 384 8.6 and 5.2; with a scale per 128-channel group the linear 50 x 1024 -> 4096 8.0 and 7.0, 5954 x 14080 -> 288
-// 233 and 223.  About 21 instructions a channel at 55% of the issue slots; neither
+// 233 and 223.  8-bit codes: the gated linear 816 x 2048 -> 2 x 16384 73.5 and 70.7, one row of 1536 -> 5168 8.5 and 7.0.  About 21 instructions a channel at 55% of the issue slots; neither
 // the transposes, the butterflies nor the conversions alone bound it (leaving one of them out saves 6 to 16%).  Staying
 // CTAs fed by TMA one group ahead were slower (73 us at 3200 x 16384): with an extra barrier a group, two CTAs an SM overlap
 // less than fresh ones.  A few rows are spread one to a CTA: 50 x 1024 2.1 us against 2.8 with eight rows a CTA; with blocks
@@ -82,9 +82,10 @@ static __device__ __noinline__ uint32_t codes4_exact(float4 y, float inv_sqrt_b,
   return (low_bytes(u[0], u[1], u[2], u[3]) & 0x0F0F0F0Fu) ^ 0x08080808u;
 }
 
-// kPacked: output packed nibbles [M][K/2] (a quad is 4 consecutive channels), else operand bytes [M][K] (each group of 8
-// stored k0 k2 k4 k6 k1 k3 k5 k7; a quad is its even or its odd channels).
-template <typename T, int kLogB, bool kStep, bool kPacked>
+// kOut, the output: 0 packed nibbles [M][K/2], 1 operand bytes [M][K]; 8-bit codes: 2 int8 rows [M][K], 3 the GEMM's two operand
+// planes [M][2 K].  In 0 and 2 a quad is 4 consecutive channels; in 1 and 3, where each group of 8 is stored k0 k2 k4 k6 k1 k3
+// k5 k7, its even or its odd ones.  8-bit codes are rounded by the other kernel's arithmetic (no E4M3 byte holds them).
+template <typename T, int kLogB, bool kStep, int kOut>
 __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(const T* __restrict__ x, int M, int K, float inv_sqrt_b,
                                                                             const float* __restrict__ step_scale,
                                                                             uint8_t* __restrict__ xq, float* __restrict__ xscale,
@@ -98,6 +99,8 @@ __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(cons
   constexpr bool kFour = kRB == 1 || kRB == 2;
   constexpr bool kHalf = kRC == 4;  // after the third phase a thread holds half quads (two channels) of 16 lines
   static_assert(kLogB <= 12, "Hadamard blocks up to 4096");
+  constexpr bool kPacked = kOut == 0, kNatural = kOut == 0 || kOut == 2, kA8 = kOut >= 2;
+  constexpr float kQ = kA8 ? 127.0f : 7.0f;
   extern __shared__ __align__(128) uint8_t wide_smem[];  // one line of 8 quads (128 bytes) per thread
   __shared__ unsigned int s_max[kWideRows], s_sum[kWideRows];
 
@@ -128,7 +131,7 @@ __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(cons
   }
   if (!one_warp) __syncthreads();  // the reduction slots are cleared before any thread adds to them
   // phase 1, leaving v as quads: quad q of the 32-channel line in v[2 q], v[2 q + 1]
-  if constexpr (kPacked) {
+  if constexpr (kNatural) {
     fwht_regs<16, 0, kA>(v);
   } else {
     // quad i0 + 2 g: the even (i0 = 0) or odd channels of group g, paired like that before the butterflies (the pair's own
@@ -235,11 +238,11 @@ __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(cons
       wm = s_max[rloc < rpc ? rloc : 0];
     }
     // max |Z| of the normalised rotation: rounding is monotone, so round(max * c) = max round(y * c)
-    delta = __fdiv_rn(__uint_as_float(wm) * inv_sqrt_b, 7.0f);
+    delta = __fdiv_rn(__uint_as_float(wm) * inv_sqrt_b, kQ);
   }
   if (active && j == 0) xscale[m] = delta;
 
-  // ---- codes: quad i of this thread as operand bytes q + 8 ----
+  // ---- codes: quad i of this thread as operand bytes q + 8 (8-bit codes: as they are) ----
   const bool zero_scale = !(delta > 0.0f);
   const float rcp = zero_scale ? 0.0f : __frcp_rn(delta);
   const bool tiny_scale = !zero_scale && isinf(rcp);  // 1 / delta overflows: plain division
@@ -251,8 +254,33 @@ __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(cons
   const float2 dn = make_float2(0.0156249701976776123046875f, 0.0156249701976776123046875f);
   uint32_t code[8];
   uint32_t sum_acc = 0;
+  if constexpr (kA8) {
+    const float2 cr2 = make_float2(cr, cr), magic2 = make_float2(kMagic, kMagic);
+    const float2 nmagic2 = make_float2(-kMagic, -kMagic), neg2 = make_float2(-1.0f, -1.0f);
 #pragma unroll
-  for (int i = 0; i < 8; i += 2) {
+    for (int i = 0; i < 8; ++i) {
+      float2 u[2];
+      float dev = 0.0f;  // the largest distance |t - round(t)| of the quad
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        float2 t = __fmul2_rn(v[2 * i + k], cr2);
+        if constexpr (kStep) t = make_float2(fminf(fmaxf(t.x, -kQ), kQ), fminf(fmaxf(t.y, -kQ), kQ));
+        u[k] = __fadd2_rn(t, magic2);
+        const float2 d = __ffma2_rn(__fadd2_rn(u[k], nmagic2), neg2, t);
+        dev = fmaxf(dev, fmaxf(fabsf(d.x), fabsf(d.y)));
+      }
+      if (dev >= kTieBand8 || tiny_scale) {  // rare: decide these values exactly
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+          u[k] = make_float2(exact_code(v[2 * i + k].x, inv_sqrt_b, delta, cr, kQ, kTieBand8),
+                             exact_code(v[2 * i + k].y, inv_sqrt_b, delta, cr, kQ, kTieBand8));
+      }
+      code[i] = low_bytes(u[0].x, u[0].y, u[1].x, u[1].y);
+      sum_acc = __dp4a(code[i] ^ 0x80808080u, 0x01010101u, sum_acc);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 8 && !kA8; i += 2) {
     uint32_t odd = 0;  // nonzero: a value near a tie, or no code
 #pragma unroll
     for (int k = i; k < i + 2; ++k) {
@@ -282,7 +310,38 @@ __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(cons
 
   // ---- store ----
   if (active) {
-    uint8_t* const dst = xq + static_cast<size_t>(m) * (kPacked ? K / 2 : K);
+    uint8_t* const dst = xq + static_cast<size_t>(m) * (kPacked ? K / 2 : kOut == 3 ? 2 * K : K);
+    // n (1, 2, 4) words of codes at channel o; the planes of a 128-code k-block are 128 bytes each, high nibbles first
+    auto put = [&](int o, auto w) {
+      using W = decltype(w);
+      if constexpr (kOut == 3) {
+        W h = w, l = w;
+#pragma unroll
+        for (int k = 0; k < static_cast<int>(sizeof(W) / 4); ++k) {
+          const uint32_t c = reinterpret_cast<const uint32_t*>(&w)[k] ^ 0x80808080u;
+          reinterpret_cast<uint32_t*>(&l)[k] = c & 0x0F0F0F0Fu;
+          reinterpret_cast<uint32_t*>(&h)[k] = hi_plane_bytes((c >> 4) & 0x0F0F0F0Fu);
+        }
+        *reinterpret_cast<W*>(dst + o + (o & ~127)) = h;
+        *reinterpret_cast<W*>(dst + o + (o & ~127) + 128) = l;
+      } else {
+        *reinterpret_cast<W*>(dst + o) = w;
+      }
+    };
+    // the two halves of a word 256 channels apart
+    auto put_halves = [&](int o, uint32_t w) {
+      if constexpr (kOut == 3) {
+        const uint32_t c = w ^ 0x80808080u, l = c & 0x0F0F0F0Fu, h = hi_plane_bytes((c >> 4) & 0x0F0F0F0Fu);
+        uint8_t* const p = dst + o + (o & ~127);
+        *reinterpret_cast<uint16_t*>(p) = static_cast<uint16_t>(h);
+        *reinterpret_cast<uint16_t*>(p + 128) = static_cast<uint16_t>(l);
+        *reinterpret_cast<uint16_t*>(p + 512) = static_cast<uint16_t>(h >> 16);
+        *reinterpret_cast<uint16_t*>(p + 640) = static_cast<uint16_t>(l >> 16);
+      } else {
+        *reinterpret_cast<uint16_t*>(dst + o) = static_cast<uint16_t>(w);
+        *reinterpret_cast<uint16_t*>(dst + o + 256) = static_cast<uint16_t>(w >> 16);
+      }
+    };
     auto nibbles = [](uint32_t w) -> uint32_t {  // four codes as two packed bytes
       const uint32_t n = w ^ 0x08080808u;
       return __byte_perm(n | (n >> 4), 0u, 0x4420);
@@ -293,8 +352,8 @@ __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(cons
             make_uint4(nibbles(code[0]) | (nibbles(code[1]) << 16), nibbles(code[2]) | (nibbles(code[3]) << 16),
                        nibbles(code[4]) | (nibbles(code[5]) << 16), nibbles(code[6]) | (nibbles(code[7]) << 16));
       } else {
-        *reinterpret_cast<uint4*>(dst + static_cast<size_t>(j) * 32) = make_uint4(code[0], code[1], code[2], code[3]);
-        *reinterpret_cast<uint4*>(dst + static_cast<size_t>(j) * 32 + 16) = make_uint4(code[4], code[5], code[6], code[7]);
+        put(j * 32, make_uint4(code[0], code[1], code[2], code[3]));
+        put(j * 32 + 16, make_uint4(code[4], code[5], code[6], code[7]));
       }
     } else if constexpr (kFour) {  // quads 2 p and 2 p + 1 of 4 lines
       const int at = j & ~3, p = j & 3;
@@ -303,7 +362,7 @@ __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(cons
         if constexpr (kPacked) {
           *reinterpret_cast<uint32_t*>(dst + (at + l) * 16 + p * 4) = nibbles(code[2 * l]) | (nibbles(code[2 * l + 1]) << 16);
         } else {
-          *reinterpret_cast<uint2*>(dst + (at + l) * 32 + p * 8) = make_uint2(code[2 * l], code[2 * l + 1]);
+          put((at + l) * 32 + p * 8, make_uint2(code[2 * l], code[2 * l + 1]));
         }
       }
     } else {
@@ -318,8 +377,7 @@ __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(cons
             dst[at * 16 + piece] = static_cast<uint8_t>(n);
             dst[(at + 8) * 16 + piece] = static_cast<uint8_t>(n >> 8);
           } else {
-            *reinterpret_cast<uint16_t*>(dst + at * 32 + piece * 2) = static_cast<uint16_t>(code[i]);
-            *reinterpret_cast<uint16_t*>(dst + (at + 8) * 32 + piece * 2) = static_cast<uint16_t>(code[i] >> 16);
+            put_halves(at * 32 + piece * 2, code[i]);
           }
           continue;
         }
@@ -333,7 +391,7 @@ __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(cons
         if constexpr (kPacked) {
           *reinterpret_cast<uint16_t*>(dst + line * 16 + q * 2) = static_cast<uint16_t>(nibbles(code[i]));
         } else {
-          *reinterpret_cast<uint32_t*>(dst + line * 32 + q * 4) = code[i];
+          put(line * 32 + q * 4, code[i]);
         }
       }
     }
@@ -345,7 +403,7 @@ __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(cons
     if (active && (j & (tg - 1)) == 0) xgsum[static_cast<size_t>(m) * (K >> gshift) + ((j * 32) >> gshift)] = gs;
   }
   if (xsum != nullptr) {
-    unsigned int cs = sum_acc - 8u * 32u;  // every code carried an offset of 8
+    unsigned int cs = sum_acc - (kA8 ? 128u : 8u) * 32u;  // every code carried an offset
     if (row_warp) {
       cs = __reduce_add_sync(0xffffffffu, cs);
       if (!one_warp && (tid & 31) == 0 && rloc < rpc) atomicAdd(&s_sum[rloc], cs);
@@ -362,7 +420,7 @@ __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(cons
   }
 }
 
-template <typename T, int kLogB, bool kStep, bool kPacked>
+template <typename T, int kLogB, bool kStep, int kOut>
 cudaError_t launch_wide_t(const RotQuantArgs& a) {
   const int tpr = a.K / 32;
   int rows = tpr >= 256 ? 1 : 256 / tpr;
@@ -370,7 +428,7 @@ cudaError_t launch_wide_t(const RotQuantArgs& a) {
   while (rows > 1 && (a.M + rows - 1) / rows < a.num_sms) rows /= 2;  // few rows: more CTAs, down to one row each
   const int tpb = (rows * tpr + 31) & ~31;  // whole warps: the warp-wide steps take every lane
   rows = tpb / tpr;                         // as the kernel counts them
-  auto kern = rotate_quant_wide_kernel<T, kLogB, kStep, kPacked>;
+  auto kern = rotate_quant_wide_kernel<T, kLogB, kStep, kOut>;
   const size_t smem = kLogB > 5 ? static_cast<size_t>(tpb) * 128 : 0;
   if (smem > 40 * 1024) {  // (48 KB without it, the kernel's own few words included)
     constexpr int kMaxSmem = kWideThreads * 128;  // raised once per device to the most any K asks of it
@@ -401,29 +459,28 @@ cudaError_t launch_wide_t(const RotQuantArgs& a) {
   return cudaGetLastError();
 }
 
-template <typename T, bool kStep, bool kPacked>
+template <typename T, bool kStep, int kOut>
 cudaError_t launch_wide_b(const RotQuantArgs& a) {
   switch (a.log_b) {
-    case 0: return launch_wide_t<T, 0, kStep, kPacked>(a);
-    case 1: return launch_wide_t<T, 1, kStep, kPacked>(a);
-    case 2: return launch_wide_t<T, 2, kStep, kPacked>(a);
-    case 3: return launch_wide_t<T, 3, kStep, kPacked>(a);
-    case 4: return launch_wide_t<T, 4, kStep, kPacked>(a);
-    case 5: return launch_wide_t<T, 5, kStep, kPacked>(a);
-    case 6: return launch_wide_t<T, 6, kStep, kPacked>(a);
-    case 7: return launch_wide_t<T, 7, kStep, kPacked>(a);
-    case 8: return launch_wide_t<T, 8, kStep, kPacked>(a);
-    case 9: return launch_wide_t<T, 9, kStep, kPacked>(a);
-    case 10: return launch_wide_t<T, 10, kStep, kPacked>(a);
-    case 11: return launch_wide_t<T, 11, kStep, kPacked>(a);
-    default: return launch_wide_t<T, 12, kStep, kPacked>(a);
+    case 0: return launch_wide_t<T, 0, kStep, kOut>(a);
+    case 1: return launch_wide_t<T, 1, kStep, kOut>(a);
+    case 2: return launch_wide_t<T, 2, kStep, kOut>(a);
+    case 3: return launch_wide_t<T, 3, kStep, kOut>(a);
+    case 4: return launch_wide_t<T, 4, kStep, kOut>(a);
+    case 5: return launch_wide_t<T, 5, kStep, kOut>(a);
+    case 6: return launch_wide_t<T, 6, kStep, kOut>(a);
+    case 7: return launch_wide_t<T, 7, kStep, kOut>(a);
+    case 8: return launch_wide_t<T, 8, kStep, kOut>(a);
+    case 9: return launch_wide_t<T, 9, kStep, kOut>(a);
+    case 10: return launch_wide_t<T, 10, kStep, kOut>(a);
+    case 11: return launch_wide_t<T, 11, kStep, kOut>(a);
+    default: return launch_wide_t<T, 12, kStep, kOut>(a);
   }
 }
 
-template <typename T>
+template <typename T, int kOut>
 cudaError_t launch_wide(const RotQuantArgs& a) {
-  if (a.out_mode == 0) return a.mode == 1 ? launch_wide_b<T, true, true>(a) : launch_wide_b<T, false, true>(a);
-  return a.mode == 1 ? launch_wide_b<T, true, false>(a) : launch_wide_b<T, false, false>(a);
+  return a.mode == 1 ? launch_wide_b<T, true, kOut>(a) : launch_wide_b<T, false, kOut>(a);
 }
 
 }  // namespace rq

@@ -171,3 +171,39 @@ def test_every_row_width_runs(K):
     codes = _unpack(xq).to(torch.int32) - 8
     assert torch.equal(codes.sum(1, dtype=torch.int32), xsum)
     assert int(codes.abs().max()) == 7
+
+
+@pytest.mark.parametrize("M,K,log_b,dt", [(m, k, b, d) for b, (m, k, d) in enumerate([
+    (200, 640, "f16"), (33, 128, "bf16"), (70, 384, "f32"), (5, 1152, "f16"), (300, 256, "bf16"), (9, 3200, "f16"),
+    (77, 2944, "bf16"), (129, 896, "f16"), (50, 2304, "f32"), (65, 1536, "f16"), (8, 3072, "bf16"), (130, 2048, "f16"),
+    (50, 4096, "bf16")])])
+def test_eight_bit_codes_of_every_block(M, K, log_b, dt):
+    """Codes within half a step of the float64 rotation (a float32 rotation's error of a step's 2^-9 added), code sums theirs, and the
+    linear's operand planes equal those made from the int8 rows (the same outputs)."""
+    had = 1 << log_b
+    rng = np.random.default_rng(K + log_b)
+    x = _values(rng, M, K, had, dt, special=False)
+    code = Q.DTYPE_CODES[dt]
+    xq = torch.full((M, K), 99, dtype=torch.int8, device=G.DEV)
+    xs = torch.empty(M, dtype=torch.float32, device=G.DEV)
+    xsum = torch.empty(M, dtype=torch.int32, device=G.DEV)
+    Q.qvla_rotate_quantize_rows_a8(x, code, M, K, had, None, xq, xs, xsum, G.stream())
+    h = torch.ones(1, 1, dtype=torch.float64)
+    for _ in range(log_b):
+        h = torch.cat((torch.cat((h, h), 1), torch.cat((h, -h), 1)), 0)
+    z = (x.double().cpu().view(M, K // had, had) @ (h / had ** 0.5)).reshape(M, K)
+    step = z.abs().amax(1) / 127
+    assert torch.allclose(xs.double().cpu(), step, rtol=1e-5, atol=0)
+    q = xq.cpu().double()
+    assert float((q - z / step[:, None]).abs().max()) <= 0.5 + 2.0 ** -9
+    assert torch.equal(xq.to(torch.int32).sum(1, dtype=torch.int32), xsum)
+    layer = Q.qvla_layer_create(32, K, had, code, Q.F16, rng.integers(0, 256, (32, K // 2), dtype=np.uint8),
+                                np.full(32, 1e-3, np.float32), None)
+    nb = Q.qvla_w4a8_workspace_bytes(layer, M)
+    work = torch.empty(nb, dtype=torch.uint8, device=G.DEV)
+    y, want = (torch.empty(M, 32, dtype=torch.float16, device=G.DEV) for _ in range(2))
+    Q.qvla_w4a8_linear(layer, x, M, -1, y, work, nb, G.stream())
+    Q.qvla_gemm_w4a8(layer, xq, xs, M, want, None, work, nb, G.stream())
+    Q.qvla_check_device(G.stream())
+    assert torch.equal(y, want)
+    layer.close()
