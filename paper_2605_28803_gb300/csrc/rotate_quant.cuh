@@ -1,15 +1,17 @@
 // Fused online rotation + symmetric int4 activation quantisation (Sec. 4.1 Eq. 3-5, the online
 // block-Hadamard factor; Sec. 4.2 Eq. 5-6 with per-token or per-step scales).
 //
+// The calibration maxima, and per-step codes in scale groups of 2048 and 4096 channels; every other call takes
+// rotate_quant_wide.cuh or rotate_quant_pass.cu, which share the helpers here.
+//
 // One row of x is spread over K/EPT threads, EPT consecutive elements each (16-byte loads),
 // held as float2 pairs.  The fast Walsh-Hadamard transform of a block of b = 2^LOGB elements
 // runs its butterfly stages on the low log2(EPT) index bits in registers (stages of distance
 // >= 2 as packed f32x2 adds/subs), then transposes once through shared memory so that each
 // thread holds the elements that differ in the remaining bits, and runs those in registers
-// too.  The scale (per token: max |y| / q_max; or the step's table entry), the codes, their
-// packing and the row's code sum follow from registers.  Codes are int4 (q_max 7) or, for the
-// W4A8 variant, int8 (q_max 127).  Instantiated per input dtype and code width in
-// rotate_quant_{f16,bf16,f32}.cu (4-bit) and rotate_quant_a8_{f16,bf16,f32}.cu (8-bit).
+// too.  The scale (per token: max |y| / 7; or the step's table entry), the codes as operand bytes
+// and the groups' code sums follow from registers.  Instantiated per input dtype in
+// rotate_quant_{f16,bf16,f32}.cu.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -134,17 +136,15 @@ __device__ __forceinline__ uint32_t sum8_offset(uint32_t w, uint32_t acc) {
 // channels, so all of a thread's elements share one group: with a per-group step table
 // (step_scale[g]) the thread takes its group's entry, xgsum (when set) receives each group's
 // code sum [M][K >> gshift], and calibration (absmax_out) raises one maximum per group.
-// kA8: 8-bit codes (q_max 127; out_mode int8 rows or the GEMM's two operand planes), else
-// 4-bit (q_max 7; packed nibbles or operand bytes).
-template <typename T, int kLogB, int kEpt, bool kStep, bool kA8>
+template <typename T, int kLogB, int kEpt, bool kStep>
 __global__ void __launch_bounds__(256) rotate_quant_kernel(const T* __restrict__ x, int M, int K, float inv_sqrt_b,
                                                              const float* __restrict__ step_scale,
                                                              uint8_t* __restrict__ xq, float* __restrict__ xscale,
                                                              int32_t* __restrict__ xsum, float* __restrict__ absmax_out,
-                                                             int out_mode, int gshift, int32_t* __restrict__ xgsum,
+                                                             int gshift, int32_t* __restrict__ xgsum,
                                                              int32_t* __restrict__ zero, int zero_n) {
-  constexpr float kQ = kA8 ? 127.0f : 7.0f;
-  constexpr float kBand = kA8 ? kTieBand8 : kTieBand;
+  constexpr float kQ = 7.0f;
+  constexpr float kBand = kTieBand;
   constexpr int kP = (kEpt == 128) ? 7 : 6;  // log2(kEpt)
   static_assert((1 << kP) == kEpt, "EPT");
   constexpr int kN = kEpt / 2;                // float2 per thread
@@ -276,10 +276,8 @@ __global__ void __launch_bounds__(256) rotate_quant_kernel(const T* __restrict__
   const float rcp = zero_scale ? 0.0f : __fdiv_rn(1.0f, delta);
   const bool tiny_scale = !zero_scale && isinf(rcp);  // 1/delta overflows: plain division
   const float cr = inv_sqrt_b * rcp;                  // y * cr ~ z / delta (0 when delta = 0: codes 0)
-  // codes in register order, 8 per word (register element r = 8 g + i)
-  // 4-bit: pk = packed nibbles; 8-bit: ev / od = the two's-complement code bytes of the even /
-  // odd elements of each group of 8
-  uint32_t pk[kA8 ? 1 : kEpt / 8], ev[kA8 ? kEpt / 8 : 1], od[kA8 ? kEpt / 8 : 1];
+  // codes in register order, 8 packed nibbles per word (register element r = 8 g + i)
+  uint32_t pk[kEpt / 8];
   uint32_t sum_acc = 0;
   const float2 cr2 = make_float2(cr, cr);
   const float2 magic2 = make_float2(kMagic, kMagic), nmagic2 = make_float2(-kMagic, -kMagic);
@@ -310,48 +308,12 @@ __global__ void __launch_bounds__(256) rotate_quant_kernel(const T* __restrict__
     // byte j of the packed word: code 8 g + 2 j (low nibble) and 8 g + 2 j + 1 (high nibble)
     const uint32_t even = low_bytes(u[0].x, u[1].x, u[2].x, u[3].x);
     const uint32_t odd = low_bytes(u[0].y, u[1].y, u[2].y, u[3].y);
-    if constexpr (kA8) {
-      ev[g] = even;
-      od[g] = odd;
-      sum_acc = __dp4a(even ^ 0x80808080u, 0x01010101u, sum_acc);  // sum of q + 128
-      sum_acc = __dp4a(odd ^ 0x80808080u, 0x01010101u, sum_acc);
-    } else {
-      pk[g] = (even & 0x0F0F0F0Fu) | ((odd << 4) & 0xF0F0F0F0u);
-      sum_acc = sum8_offset(pk[g], sum_acc);
-    }
+    pk[g] = (even & 0x0F0F0F0Fu) | ((odd << 4) & 0xF0F0F0F0u);
+    sum_acc = sum8_offset(pk[g], sum_acc);
   }
 
   // ---- store: run r holds register elements [r kRun, (r + 1) kRun), contiguous in the row ----
-  if constexpr (!kA8) {
-  if (active && out_mode == 0) {  // packed nibbles [M][K/2]
-    uint8_t* dst = xq + static_cast<size_t>(m) * (K / 2);
-#pragma unroll
-    for (int run = 0; run < kEpt / kRun; ++run) {
-      int e0;  // first element of this run within the row
-      if constexpr (kPhase2) {
-        e0 = ((j >> kR) << kLogB) | (run << kP) | ((j & ((1 << kR) - 1)) << kL);
-      } else {
-        e0 = j * kEpt;
-      }
-      uint8_t* p = dst + (e0 >> 1);
-      constexpr int kBytes = kRun / 2;
-      const int b0 = run * kBytes;  // first byte of the run in pk
-      if constexpr (kBytes == 1) {
-        *p = static_cast<uint8_t>(pk[b0 >> 2] >> (8 * (b0 & 3)));
-      } else if constexpr (kBytes == 2) {
-        *reinterpret_cast<uint16_t*>(p) = static_cast<uint16_t>(pk[b0 >> 2] >> (8 * (b0 & 3)));
-      } else if constexpr (kBytes == 4) {
-        *reinterpret_cast<uint32_t*>(p) = pk[b0 >> 2];
-      } else if constexpr (kBytes == 8) {
-        *reinterpret_cast<uint2*>(p) = make_uint2(pk[b0 >> 2], pk[(b0 >> 2) + 1]);
-      } else {
-#pragma unroll
-        for (int w = 0; w < kBytes / 4; w += 4)
-          *reinterpret_cast<uint4*>(p + 4 * w) =
-              make_uint4(pk[(b0 >> 2) + w], pk[(b0 >> 2) + w + 1], pk[(b0 >> 2) + w + 2], pk[(b0 >> 2) + w + 3]);
-      }
-    }
-  } else if (active) {
+  if (active) {
     // One byte per code, the GEMM's tensor-core operand encoding: code q as the E4M3 byte
     // q + 8 (= q XOR 8).  Within each group of 8 consecutive k the bytes are stored in the order
     // k0 k2 k4 k6 k1 k3 k5 k7 -- the order the GEMM gives the packed operand it expands -- so
@@ -390,81 +352,14 @@ __global__ void __launch_bounds__(256) rotate_quant_kernel(const T* __restrict__
       }
     }
   }
-  }  // 4-bit
-  if constexpr (kA8) {
-    if (active) {
-#pragma unroll
-      for (int run = 0; run < kEpt / kRun; ++run) {
-        int e0;  // first element of this run within the row
-        if constexpr (kPhase2) {
-          e0 = ((j >> kR) << kLogB) | (run << kP) | ((j & ((1 << kR) - 1)) << kL);
-        } else {
-          e0 = j * kEpt;
-        }
-        if (out_mode == 2) {
-          // int8 codes [M][K], natural order
-          int8_t* dst = reinterpret_cast<int8_t*>(xq) + static_cast<size_t>(m) * K + e0;
-          if constexpr (kRun >= 8) {
-#pragma unroll
-            for (int t = 0; t < kRun / 8; ++t) {
-              const int w = run * (kRun / 8) + t;
-              *reinterpret_cast<uint2*>(dst + 8 * t) =
-                  make_uint2(__byte_perm(ev[w], od[w], 0x5140), __byte_perm(ev[w], od[w], 0x7362));
-            }
-          } else if constexpr (kRun == 4) {  // elements 4 h .. 4 h + 3 of group w
-            const int w = run >> 1, h = run & 1;
-            *reinterpret_cast<uint32_t*>(dst) = h ? __byte_perm(ev[w], od[w], 0x7362) : __byte_perm(ev[w], od[w], 0x5140);
-          } else {  // kRun == 2: elements 2 q, 2 q + 1 of group w
-            const int w = run >> 2, q = run & 3;
-            *reinterpret_cast<uint16_t*>(dst) =
-                static_cast<uint16_t>(((ev[w] >> (8 * q)) & 0xFFu) | (((od[w] >> (8 * q)) & 0xFFu) << 8));
-          }
-        } else {
-          // the GEMM's two operand planes [M][2K]: per k-block of 128 codes, 128 bytes of the
-          // high nibbles (E4M3 of v 2^-5) then 128 of the low nibbles (E4M3 of v 2^-9), each
-          // group of 8 in the order k0 k2 k4 k6 k1 k3 k5 k7; nibbles of q + 128
-          uint8_t* hp = xq + static_cast<size_t>(m) * (2 * K) + 2 * (e0 & ~127) + ((e0 & 127) & ~7);
-          uint8_t* lp = hp + 128;
-          auto planes = [&](int w, uint32_t& he, uint32_t& ho, uint32_t& le, uint32_t& lo) {
-            a8_planes(ev[w], od[w], he, ho, le, lo);
-          };
-          if constexpr (kRun >= 8) {
-#pragma unroll
-            for (int t = 0; t < kRun / 8; ++t) {
-              uint32_t he, ho, le, lo;
-              planes(run * (kRun / 8) + t, he, ho, le, lo);
-              *reinterpret_cast<uint2*>(hp + 8 * t) = make_uint2(he, ho);
-              *reinterpret_cast<uint2*>(lp + 8 * t) = make_uint2(le, lo);
-            }
-          } else if constexpr (kRun == 4) {  // elements o .. o + 3 (o = 4 h) of a group
-            const int w = run >> 1, h = run & 1, o = e0 & 7;
-            uint32_t he, ho, le, lo;
-            planes(w, he, ho, le, lo);
-            *reinterpret_cast<uint16_t*>(hp + (o >> 1)) = static_cast<uint16_t>(he >> (16 * h));
-            *reinterpret_cast<uint16_t*>(hp + 4 + (o >> 1)) = static_cast<uint16_t>(ho >> (16 * h));
-            *reinterpret_cast<uint16_t*>(lp + (o >> 1)) = static_cast<uint16_t>(le >> (16 * h));
-            *reinterpret_cast<uint16_t*>(lp + 4 + (o >> 1)) = static_cast<uint16_t>(lo >> (16 * h));
-          } else {  // kRun == 2: elements o, o + 1 (o = 2 q)
-            const int w = run >> 2, q = run & 3, o = e0 & 7;
-            uint32_t he, ho, le, lo;
-            planes(w, he, ho, le, lo);
-            hp[o >> 1] = static_cast<uint8_t>(he >> (8 * q));
-            hp[4 + (o >> 1)] = static_cast<uint8_t>(ho >> (8 * q));
-            lp[o >> 1] = static_cast<uint8_t>(le >> (8 * q));
-            lp[4 + (o >> 1)] = static_cast<uint8_t>(lo >> (8 * q));
-          }
-        }
-      }
-    }
-  }
   if (xgsum != nullptr) {  // the code sum of each scale group of the row (tg consecutive lanes)
-    int gs = static_cast<int>(sum_acc) - (kA8 ? 128 : 8) * kEpt;
+    int gs = static_cast<int>(sum_acc) - 8 * kEpt;
     const int tg = (1 << gshift) / kEpt;
     for (int o = tg >> 1; o > 0; o >>= 1) gs += __shfl_xor_sync(0xffffffffu, gs, o);
     if (active && (j & (tg - 1)) == 0) xgsum[static_cast<size_t>(m) * (K >> gshift) + grp] = gs;
   }
   if (xsum != nullptr) {
-    int cs = static_cast<int>(sum_acc) - (kA8 ? 128 : 8) * kEpt;  // every code carried an offset
+    int cs = static_cast<int>(sum_acc) - 8 * kEpt;  // every code carried an offset
     if ((tpr & 31) == 0) {
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) cs += __shfl_xor_sync(0xffffffffu, cs, o);
@@ -480,7 +375,7 @@ __global__ void __launch_bounds__(256) rotate_quant_kernel(const T* __restrict__
   }
 }
 
-template <typename T, int kLogB, bool kStep, bool kA8>
+template <typename T, int kLogB, bool kStep>
 cudaError_t launch_t(const RotQuantArgs& a) {
   constexpr int kEpt = kLogB >= 12 ? 128 : 64;
   const int tpr = a.K / kEpt;
@@ -490,7 +385,7 @@ cudaError_t launch_t(const RotQuantArgs& a) {
   const int grid = (a.M + rows - 1) / rows;
   if (grid == 0) return cudaSuccess;
   const size_t smem = (kLogB > ((kEpt == 128) ? 7 : 6)) ? static_cast<size_t>(tpb) * kEpt * sizeof(float) : 0;
-  auto kern = rotate_quant_kernel<T, kLogB, kEpt, kStep, kA8>;
+  auto kern = rotate_quant_kernel<T, kLogB, kEpt, kStep>;
   if (smem > 40 * 1024) {  // (48 KB without it, the kernel's own few words included: K = 12288 needs it)
     // raise the kernel's limit once per device to the most any K asks of it (one kernel serves
     // several K, so several sizes: at most 256 threads x 128 float32 = 128 KB)
@@ -518,36 +413,35 @@ cudaError_t launch_t(const RotQuantArgs& a) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   cudaError_t e = cudaLaunchKernelEx(&cfg, kern, reinterpret_cast<const T*>(a.x), a.M, a.K, a.inv_sqrt_b, a.step_scale,
-                                     a.xq, a.xscale, a.xsum, a.mode == 2 ? a.absmax : nullptr, a.out_mode,
+                                     a.xq, a.xscale, a.xsum, a.mode == 2 ? a.absmax : nullptr,
                                      a.gshift, a.xgsum, a.zero, a.zero_n);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
 
-template <typename T, bool kStep, bool kA8>
+template <typename T, bool kStep>
 cudaError_t launch_mode(const RotQuantArgs& a) {
   switch (a.log_b) {
-    case 0: return launch_t<T, 0, kStep, kA8>(a);
-    case 1: return launch_t<T, 1, kStep, kA8>(a);
-    case 2: return launch_t<T, 2, kStep, kA8>(a);
-    case 3: return launch_t<T, 3, kStep, kA8>(a);
-    case 4: return launch_t<T, 4, kStep, kA8>(a);
-    case 5: return launch_t<T, 5, kStep, kA8>(a);
-    case 6: return launch_t<T, 6, kStep, kA8>(a);
-    case 7: return launch_t<T, 7, kStep, kA8>(a);
-    case 8: return launch_t<T, 8, kStep, kA8>(a);
-    case 9: return launch_t<T, 9, kStep, kA8>(a);
-    case 10: return launch_t<T, 10, kStep, kA8>(a);
-    case 11: return launch_t<T, 11, kStep, kA8>(a);
-    case 12: return launch_t<T, 12, kStep, kA8>(a);
+    case 0: return launch_t<T, 0, kStep>(a);
+    case 1: return launch_t<T, 1, kStep>(a);
+    case 2: return launch_t<T, 2, kStep>(a);
+    case 3: return launch_t<T, 3, kStep>(a);
+    case 4: return launch_t<T, 4, kStep>(a);
+    case 5: return launch_t<T, 5, kStep>(a);
+    case 6: return launch_t<T, 6, kStep>(a);
+    case 7: return launch_t<T, 7, kStep>(a);
+    case 8: return launch_t<T, 8, kStep>(a);
+    case 9: return launch_t<T, 9, kStep>(a);
+    case 10: return launch_t<T, 10, kStep>(a);
+    case 11: return launch_t<T, 11, kStep>(a);
+    case 12: return launch_t<T, 12, kStep>(a);
     default: return cudaErrorInvalidValue;
   }
 }
 
-// kA8: the 8-bit instantiations (out_mode 2 or 3), compiled in translation units of their own.
-template <typename T, bool kA8>
+template <typename T>
 cudaError_t launch_dtype(const RotQuantArgs& a) {
-  return a.mode == 1 ? launch_mode<T, true, kA8>(a) : launch_mode<T, false, kA8>(a);
+  return a.mode == 1 ? launch_mode<T, true>(a) : launch_mode<T, false>(a);
 }
 
 }  // namespace rq
