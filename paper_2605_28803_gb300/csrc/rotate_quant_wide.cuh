@@ -1,5 +1,5 @@
-// Fused online rotation + symmetric 4-bit activation quantisation (Sec. 4.1 Eq. 3-5, Sec. 4.2 Eq. 5-6) for batches of rows:
-// 32 channels per thread, 4-bit codes by packed E4M3 conversion, 8-bit codes by magic-number rounding.
+// Fused online rotation + symmetric 4-bit or 8-bit activation quantisation (Sec. 4.1 Eq. 3-5, Sec. 4.2 Eq. 5-6) for batches of
+// rows: 32 channels per thread, 4-bit codes by packed E4M3 conversion, 8-bit codes by magic-number rounding.
 //
 // It does what rotate_quant.cuh's kernel does, bit for bit, with fewer instructions
 // per channel and twice the warps in flight:
