@@ -37,18 +37,6 @@ __device__ __forceinline__ bool elect_one() {
 // The warp's index in its block, as a value the compiler knows to be the same in every lane.
 __device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, static_cast<int>(threadIdx.x >> 5), 0); }
 
-// 2^x and 1 / x to about one ulp; subnormal results are zero.
-__device__ __forceinline__ float exp2_approx(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ float rcp_approx(float x) {
-  float y;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 // Register split between warpgroups (every warp of a warpgroup executes it once): the registers a thread may use from
 // here on.  An increase waits until the block's other warpgroups have given enough up.
 template <int kRegs>
