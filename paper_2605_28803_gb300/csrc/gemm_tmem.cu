@@ -275,8 +275,11 @@ __global__ void __launch_bounds__(kTmThreads, 1) gemm_tmem_kernel(const __grid_c
             const uint32_t b = (desc_lo | (b0 >> 4)) + static_cast<uint32_t>(kPacked ? sa : s) * b_stage;
 #pragma unroll
             for (int h = 0; h < kKb; ++h) {
-              const bool real = h == 0 || kb + h < kz;  // a unit's last stage may hold one k-block: its release only
-              if (real && !__all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_full[s][h]), ph))) { ok = false; break; }
+              // A unit's last stage may hold one k-block.  The converters fill and announce its second one all the same
+              // (bytes that no MMA reads): it is waited for before it is released, or a late store of theirs could land
+              // on the slot's next weights, which with an odd SA other warps write.
+              const bool real = h == 0 || kb + h < kz;
+              if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bar_full[s][h]), ph))) { ok = false; break; }
               tc_fence_after();
               const uint32_t empty = smem_u32(&bar_empty[s][h]);
               if (elect_one()) {

@@ -101,6 +101,47 @@ def test_packed_codes_equal_slices_of_few_tokens(M, K, N, gated, dt):
     layer.close()
 
 
+@pytest.mark.parametrize("packed,M,K,N,gated", [
+    (False, 485, 384, 19968, False), (False, 202, 896, 13312, False), (False, 199, 1152, 13056, False),
+    (False, 131, 384, 21760, False), (False, 129, 1152, 21248, False), (False, 36, 384, 19968, True),
+    (False, 33, 1152, 12288, True), (False, 99, 896, 10496, True), (False, 129, 896, 10496, True),
+    (True, 195, 384, 19712, False), (True, 194, 1152, 20224, False), (True, 39, 384, 20480, True),
+    (True, 34, 1664, 11264, True), (True, 99, 1152, 20224, True)])
+def test_odd_k_blocks_over_several_tiles_a_pair(packed, M, K, N, gated):
+    """An odd number of k-blocks leaves a tile's last ring stage half filled, and the next tile of the pair takes the same
+    TMEM slots an odd number of stages later (3 at 128- and 160-token tiles, 5 at 64), from other converter warps.  Every run
+    must be the bits of slices of a few tokens, on the weight-major kernel or, gated, the GEMV."""
+    rng = np.random.default_rng(M + K + N)
+    layer, _ = _layer(rng, N, K, 128, "f16", gated)
+    y = torch.empty(M, N, dtype=torch.float16, device=G.DEV)
+    if packed:
+        q = rng.integers(-7, 8, (M, K)).astype(np.int8)
+        xq = torch.from_numpy(O.pack_int4(q)).to(G.DEV)
+        xsum = torch.from_numpy(q.sum(1, dtype=np.int32)).to(G.DEV)
+        xs = torch.from_numpy(rng.uniform(0.5, 1.5, M).astype(np.float32) / 64).to(G.DEV)
+
+        def run(i, m, out):
+            Q.qvla_gemm_w4a4(layer, xq[i:], xs[i : i + m].clone(), xsum[i : i + m].clone(), m, out, None, G.stream())
+    else:
+        x = torch.from_numpy(rng.standard_normal((M, K), dtype=np.float32)).half().to(G.DEV)
+        nb = Q.qvla_linear_workspace_bytes(layer, M)
+        work = torch.empty(nb, dtype=torch.uint8, device=G.DEV)
+
+        def run(i, m, out):
+            Q.qvla_w4a4_linear(layer, x[i:], m, -1, out, work, nb, G.stream())
+
+    rows = 4 if gated else 128
+    want = torch.empty_like(y)
+    for i in range(0, M, rows):
+        run(i, min(rows, M - i), want[i:])
+    for _ in range(20):
+        y.fill_(float("nan"))
+        run(0, M, y)
+        assert torch.equal(y, want)
+    Q.qvla_check_device(G.stream())
+    layer.close()
+
+
 @pytest.mark.parametrize("M,K,N,gated", [(200, 1152, 272, False), (129, 128, 16, False), (77, 896, 256, True)])
 def test_eight_bit_codes_give_the_oracles_integers(M, K, N, gated):
     rng = np.random.default_rng(M + K)
