@@ -162,9 +162,10 @@ __device__ __forceinline__ bool rotate_quantize_token(const GvParams& p, const X
       const int e = t + 256 * w, kk = c * C + e - k0;
       m8[w] = (e < C && (whole_row || (kk >= 0 && kk < range))) ? fabsf(yp[w]) : 0.0f;
     }
-    mx = fmaxf(mx, fmaxf(fmaxf(fmaxf(m8[0], m8[1]), fmaxf(m8[2], m8[3])), fmaxf(fmaxf(m8[4], m8[5]), fmaxf(m8[6], m8[7]))));
+    using rq::max_nan;
+    mx = max_nan(mx, max_nan(max_nan(max_nan(m8[0], m8[1]), max_nan(m8[2], m8[3])), max_nan(max_nan(m8[4], m8[5]), max_nan(m8[6], m8[7]))));
   }
-  // the CTA's largest |value| (non-negative floats order as their bit patterns): one per warp
+  // the CTA's largest |value| (non-negative floats order as their bit patterns, NaN above infinity): one per warp
   const uint32_t wmax = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));
   if (lane == 0) s_wmax[warp] = wmax;
   __syncthreads();

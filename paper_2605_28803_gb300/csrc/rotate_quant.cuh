@@ -98,6 +98,14 @@ __device__ __forceinline__ void fwht_regs(float2 (&v)[kN]) {
   }
 }
 
+// The larger of two values, NaN if either is: a row's maximum takes it, so that a NaN anywhere in a row makes the row's
+// scale NaN, and with it the linear's outputs of that token (fmaxf would drop it, and the row would come out finite).
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
 // The exact decision for one value (rare: only near a tie, or when 1/delta overflows): round
 // half to even of the exact quotient z / delta for z = float32(y * c), by the sign of
 // z - h delta (one FMA is exact in sign) at the half-integer h next to t, then the clamp to

@@ -133,9 +133,9 @@ __global__ void __launch_bounds__(kRqpThreads) rotate_quant_pass_kernel(RqpParam
     }
   }
 
-  // the pass's largest |value| (non-negative floats order as their bit patterns), then the row's
-  const float mx = fmaxf(fmaxf(fmaxf(fabsf(yv[0]), fabsf(yv[1])), fmaxf(fabsf(yv[2]), fabsf(yv[3]))),
-                         fmaxf(fmaxf(fabsf(yv[4]), fabsf(yv[5])), fmaxf(fabsf(yv[6]), fabsf(yv[7]))));
+  // the pass's largest |value| (non-negative floats order as their bit patterns, NaN above infinity), then the row's
+  const float mx = rq::max_nan(rq::max_nan(rq::max_nan(fabsf(yv[0]), fabsf(yv[1])), rq::max_nan(fabsf(yv[2]), fabsf(yv[3]))),
+                               rq::max_nan(rq::max_nan(fabsf(yv[4]), fabsf(yv[5])), rq::max_nan(fabsf(yv[6]), fabsf(yv[7]))));
   const uint32_t wmax = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));
   if (lane == 0) s_wmax[warp] = wmax;
   __syncthreads();

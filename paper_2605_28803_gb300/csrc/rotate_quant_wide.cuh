@@ -223,8 +223,8 @@ __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(cons
   } else {
     float w = 0.0f;
 #pragma unroll
-    for (int i = 0; i < 16; ++i) w = fmaxf(w, fmaxf(fabsf(v[i].x), fabsf(v[i].y)));
-    unsigned int wm = __float_as_uint(w);  // non-negative floats order as their bit patterns
+    for (int i = 0; i < 16; ++i) w = max_nan(w, max_nan(fabsf(v[i].x), fabsf(v[i].y)));
+    unsigned int wm = __float_as_uint(w);  // non-negative floats order as their bit patterns, NaN above infinity
     if (row_warp) {
       wm = __reduce_max_sync(0xffffffffu, wm);
       if (!one_warp && (tid & 31) == 0 && rloc < rpc) atomicMax(&s_max[rloc], wm);

@@ -85,18 +85,39 @@ def test_a_batch_equals_the_pass_kernel_on_repeated_rows(M, K, had, dt, r):
         ob, xs, xsum = _quantise(layer, x, step)
         parts = [_quantise(wide, xr[i : i + 48], step) for i in range(0, M, 48)] if r > 1 or M > 48 else []
         want = [torch.cat(p) for p in zip(*parts)]
-        rows = torch.ones(M, dtype=torch.bool)
-        if step < 0 and M > 5:
-            # the row with a NaN: a whole block may be NaN, and the pass kernel's threads of 8 NaN values make the row's
-            # maximum NaN where this kernel's (like the 64-channel one's) leaves them out
-            rows[5] = False
-        assert torch.equal(ob.repeat(1, r)[rows], want[0][rows])
-        assert torch.equal(xs[rows], want[1][rows]) and torch.equal(r * xsum[rows], want[2][rows])
+        assert torch.equal(ob.repeat(1, r), want[0])
+        assert torch.equal(xs, want[1]) and torch.equal(r * xsum, want[2])
         scale = None if step < 0 else torch.tensor([table[step]], device=G.DEV)
         xq, pxs, pxsum = _packed(x, had, scale)
         assert torch.equal(_unpack(xq), ob) and torch.equal(pxs, xs) and torch.equal(pxsum, xsum)
     layer.close()
     wide.close()
+
+
+@pytest.mark.parametrize("xdt,ydt", [("bf16", "bf16"), ("f16", "f16"), ("f32", "f16")])
+@pytest.mark.parametrize("K,had", [(128, 1), (640, 128), (2048, 2048), (4096, 16), (4096, 4096), (6144, 2048), (16384, 1), (16384, 2048)])
+def test_a_nan_token_gives_a_nan_row(K, had, xdt, ydt):
+    """One NaN channel of a token under a scale per token makes its scale NaN and its outputs NaN, on every kernel that
+    quantises (one launch at one token, the passes, 32 channels a thread, 8-bit codes); the other tokens' outputs stay."""
+    rng = np.random.default_rng(K + had)
+    N = 32
+    layer = Q.qvla_layer_create(N, K, had, Q.DTYPE_CODES[xdt], Q.DTYPE_CODES[ydt], rng.integers(0, 256, (N, K // 2), dtype=np.uint8),
+                                np.full(N, 1e-3, np.float32), rng.standard_normal(N).astype(np.float32))
+    for M in (1, 2, 4, 33, 50, 64, 65, 200):
+        x = torch.from_numpy(rng.standard_normal((M, K)).astype(np.float32)).to(_T[xdt]).to(G.DEV)
+        bad = x.clone()
+        bad[M // 2, int(rng.integers(K))] = np.nan
+        nb = max(Q.qvla_linear_workspace_bytes(layer, M), Q.qvla_w4a8_workspace_bytes(layer, M))
+        work = torch.empty(nb, dtype=torch.uint8, device=G.DEV)
+        for linear in (Q.qvla_w4a4_linear,) + ((Q.qvla_w4a8_linear,) if K <= 4096 else ()):
+            y, want = (torch.zeros(M, N, dtype=_T[ydt], device=G.DEV) for _ in range(2))
+            linear(layer, bad, M, -1, y, work, nb, G.stream())
+            linear(layer, x, M, -1, want, work, nb, G.stream())
+            Q.qvla_check_device(G.stream())
+            want[M // 2] = np.nan
+            assert torch.equal(y.isnan(), want.isnan())
+            assert torch.equal(y[~y.isnan()], want[~want.isnan()])
+    layer.close()
 
 
 @pytest.mark.parametrize("M,K,had", [(67, 2304, 256), (131, 1024, 1024), (70, 4096, 2048), (65, 384, 32), (33, 8192, 4096),
