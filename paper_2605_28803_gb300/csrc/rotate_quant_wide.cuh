@@ -247,7 +247,9 @@ __global__ void __launch_bounds__(kWideThreads, 2) rotate_quant_wide_kernel(cons
   const float rcp = zero_scale ? 0.0f : __frcp_rn(delta);
   const bool tiny_scale = !zero_scale && isinf(rcp);  // 1 / delta overflows: plain division
   const float cr = inv_sqrt_b * rcp;                  // y * cr ~ z / delta (0 when delta = 0: codes 0)
-  const bool plain = !(cr >= 1e-30f && cr <= 1e30f);  // the scaled product below could lose bits
+  // the scaled product below could lose bits (a zero cannot: a row of zeros, such as padding, stays on the fast path, where
+  // its codes are 0 exactly; sent the other way, 3200 x 16384 f16 zeros took 76 us)
+  const bool plain = cr != 0.0f && !(cr >= 1e-30f && cr <= 1e30f);
   const float2 cr9 = make_float2(cr * 0.001953125f, cr * 0.001953125f);
   // (8 +- 2^-16) 2^-9
   const float2 up = make_float2(0.0156250298023223876953125f, 0.0156250298023223876953125f);
