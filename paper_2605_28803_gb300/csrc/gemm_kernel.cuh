@@ -136,6 +136,17 @@ struct Params {
 __device__ __forceinline__ void epi_sync() {
   asm volatile("bar.sync %0, %1;" ::"n"(kEpiBarrier), "n"(kEpiThreads) : "memory");
 }
+// The same barrier; every thread learns whether any of them came with `late` set.  The barrier itself carries the answer: read
+// from a flag in shared memory after it, it could already be that of a faster thread's next wait.
+__device__ __forceinline__ bool epi_sync_any(bool late) {
+  uint32_t any;
+  asm volatile(
+      "{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\nbar.red.or.pred q, %2, %3, p;\nselp.u32 %0, 1, 0, q;\n}\n"
+      : "=r"(any)
+      : "r"(static_cast<uint32_t>(late)), "n"(kEpiBarrier), "n"(kEpiThreads)
+      : "memory");
+  return any != 0;
+}
 
 // Expand one 16-byte chunk (32 codes) into 32 E4M3 bytes at row + the two swizzled 16-byte
 // columns o0 and o1 of a 128-byte-swizzled tile row.  The byte order inside each group of 8
@@ -416,7 +427,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w4a4_kernel(const __grid_con
   __shared__ __align__(8) uint64_t bar_xready;  // fused: this CTA's operand tile is complete
   __shared__ int s_xs[kFused ? kBN : 1];        // fused: code sums of each token over this CTA's k-range
   __shared__ uint32_t s_tmem_base;
-  __shared__ int s_epi_abort;  // set by an epilogue thread whose wait timed out
+  __shared__ int s_epi_abort;  // set by an epilogue thread whose wait timed out, for the reduction after the roles' end
   // per-column parameters of the current tile (non-swap): weight scale, code correction, bias
   __shared__ __align__(16) float s_ws[kSwap ? 1 : kBN];
   __shared__ __align__(16) float s_wc[kSwap ? 1 : kBN];
@@ -803,6 +814,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w4a4_kernel(const __grid_con
     // ------------------------------------------------------------------ epilogue
     const int et = threadIdx.x;  // 0..127 = TMEM lane
     int tile_iter = 0;
+    bool late = false;  // a wait of this thread has run out
     const float k64 = p.kconst;
     griddep_wait();  // xscale / xsum come from the previous kernel, and y may still be read by it
     if constexpr (kFused) {
@@ -826,7 +838,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w4a4_kernel(const __grid_con
         }
         s_xs[et] = (landed && et < p.M) ? static_cast<int>(sum) - 8 * (kb1 - kb0) * kBK : 0;
       }
-      if (!landed) s_epi_abort = 1;
+      if (!landed) {
+        s_epi_abort = 1;
+        late = true;
+      }
       epi_sync();
     }
     if constexpr (kGroup) {
@@ -838,8 +853,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w4a4_kernel(const __grid_con
       int gi = 0;
       for (int tile = QVLA_UNIT0; tile < ntiles; tile += QVLA_NUNITS) {
         const int ta = tile % tiles_a, tb = tile / tiles_a;
-        epi_sync();
-        if (s_epi_abort) break;
+        if (epi_sync_any(late)) break;
         if constexpr (!kSwap) {
           for (int c = et; c < kBN; c += kEpiThreads) {
             const int n = min(tb * kBN + c, p.N - 1);
@@ -870,10 +884,14 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w4a4_kernel(const __grid_con
             f_w = __ldg(wg + g + 1);
             f_x = __ldg(xg + g + 1);
           }
-          epi_sync();  // the column corrections are there, and those of two groups ago no longer read
-          if (s_epi_abort) break;
+          // the column corrections are there, and those of two groups ago no longer read
+          if (epi_sync_any(late)) {
+            late = true;
+            break;
+          }
           if (!mbar_wait(smem_u32(&bar_tfull[buf]), static_cast<uint32_t>(gi >> 1) & 1u)) {
-            s_epi_abort = 1;  // every thread leaves after the next barrier
+            s_epi_abort = 1;
+            late = true;  // every thread leaves at the next barrier
             continue;
           }
           tc_fence_after();
@@ -951,8 +969,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w4a4_kernel(const __grid_con
       // All epilogue threads pass this barrier every tile, so the abort decision below is
       // uniform and no thread is left waiting at a named barrier.  It also tells the writers
       // of the column parameters that the previous tile's readers are done.
-      epi_sync();
-      if (s_epi_abort) break;
+      if (epi_sync_any(late)) break;
       if constexpr (!kSwap) {
         // stage this tile's column parameters while the accumulator is still being computed
         for (int c = et; c < kBN; c += kEpiThreads) {
@@ -965,6 +982,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_w4a4_kernel(const __grid_con
       }
       if (!mbar_wait(smem_u32(&bar_tfull[buf]), aph)) {
         s_epi_abort = 1;
+        late = true;
         continue;
       }
       tc_fence_after();

@@ -50,6 +50,40 @@ def test_a_wait_that_runs_out_reports_timeout_and_the_next_launch_is_clean():
     layer.close()
 
 
+@pytest.mark.parametrize("M,N", [(200, 512), (50, 20480)])
+def test_a_grouped_gemm_wait_that_runs_out(M, N):
+    """One scale per step and group: the epilogue waits once a group, and all its threads leave at the same barrier, in
+    whole tiles of both orientations (token-major; weight-major with several tiles a CTA, so without a cluster)."""
+    rng = np.random.default_rng(73 + M)
+    K = 512
+    layer = G.make_layer(rng.integers(0, 256, (N, K // 2), dtype=np.uint8), np.full(N, 2 ** -9, np.float32), 64, "f16", "f16")
+    Q.qvla_set_step_group_scales(layer, rng.uniform(0.1, 0.5, (1, K // 128)).astype(np.float32))
+    x = torch.from_numpy(rng.standard_normal((M, K), dtype=np.float32)).half().to(G.DEV)
+    nbytes = Q.qvla_linear_workspace_bytes(layer, M)
+    work = torch.empty(nbytes, dtype=torch.uint8, device=G.DEV)
+
+    def run():
+        y = torch.full((M, N), float("nan"), dtype=torch.float16, device=G.DEV)
+        Q.qvla_w4a4_linear(layer, x, M, 0, y, work, nbytes, G.stream())
+        return y
+
+    y0 = run()
+    Q.qvla_check_device(G.stream())
+    assert not torch.isnan(y0).any()
+    Q.qvla_debug_set_hooks(20_000_000, True)
+    try:
+        y = run()
+        with pytest.raises(Q.QvlaError) as e:
+            Q.qvla_check_device(G.stream())
+        assert e.value.status == 6
+        assert torch.isnan(y).all().item()
+    finally:
+        Q.qvla_debug_set_hooks(0, False)
+    Q.qvla_check_device(G.stream())
+    assert torch.equal(run(), y0)
+    layer.close()
+
+
 @pytest.mark.parametrize("M", [1, 2])
 def test_a_decode_gemv_wait_that_runs_out(M):
     """The decode GEMV split over a cluster of CTAs: with the hook, no CTA sends its row maximum
