@@ -29,19 +29,19 @@ extern "C" {
  * again. */
 qvla_status qvla_debug_set_hooks(unsigned long long wait_limit_ns, int hold_gemm_loads);
 
-/* The token-major GEMM's estimate (Sec. 4.2, Eq. 7) for M > 128 tokens of an M x K -> N layer on a
- * device of num_sms SMs: the tile shape and split of K with the least estimated time, computed
- * without touching a device.  The dispatch weighs it against the CTA-pair kernel with the weights in
- * TMEM, which takes qvla_w4a4_linear's GEMM from K = 768 on and plans its own tiles and split; below,
- * and for packed codes, the token-major kernel runs the shape in whole tiles where it is faster.
+/* The launch of qvla_w4a4_linear's GEMM (Sec. 4.2, Eq. 7; one scale per token or step) for M > 128
+ * tokens of an M x K -> N layer on a device of num_sms SMs: the kernel, its tile shape and its split
+ * of K, computed without touching a device.
  *   N          the layer's weight rows (2H for a gated layer)
  *   gated      nonzero: a gated gate/up layer (qvla_layer_create_gated)
  *   split_room nonzero: the workspace has the room qvla_linear_workspace_bytes counts for the
  *              split of K; 0: the linear runs in a workspace of the required parts only
- *   shape      out: 0 single CTAs with 128 x 128 tiles, 1 single CTAs with 128 x 256, 2 CTA pairs
- *              with 256 x 128, 3 CTA pairs with 256 x 256 (tokens x weight rows)
+ *   shape      out: the token-major kernel's 0 single CTAs with 128 x 128 tiles, 1 single CTAs with
+ *              128 x 256 (2 and 3: CTA pairs with 256 x 128 and 256 x 256, which it takes for packed
+ *              codes only); 3 + i, i from 1 to 6: CTA pairs with the weights in TMEM, tiles of 32 i x
+ *              256 (tokens x weight rows)
  *   parts      out: work units per tile; 1 = whole tiles
- * QVLA_ERR_INVALID_ARG for null outputs, M <= 128 (those batches run weight-major), K not a
+ * QVLA_ERR_INVALID_ARG for null outputs, M <= 128 (those batches run other kernels), K not a
  * positive multiple of 128, N not a positive multiple of 16 (256 when gated), num_sms < 2. */
 qvla_status qvla_debug_gemm_plan(int M, int K, int N, int gated, int num_sms, int split_room, int* shape, int* parts);
 

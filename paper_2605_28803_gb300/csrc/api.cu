@@ -652,9 +652,10 @@ size_t workspace_min(const qvla_layer* L, int M) {
          round256(static_cast<size_t>(M) * L->G * 4) + (L->rblock ? round256(rotated_bytes(L, M)) : 0);
 }
 constexpr int kMaxParts = 4;  // work units per tile of the GEMM's split of K
-// The GEMM's split of K: a non-gated token-major layer (M > 128) whose 128 x 256 tiles leave SMs
-// idle may split; room for kMaxParts FP32 partials of every output (rows and weight rows padded to
-// 256) and a count for each 128 x 128 tile covers every tile shape it can take.
+// The GEMM's split of K (gemm_tmem.cu): a non-gated layer of more than 128 tokens whose 128 x 256 tiles leave SMs idle may
+// split; there is room for kMaxParts FP32 partials of every output (rows and weight rows padded to 256) and a count for each
+// 128 x 128 tile.  A tile of w tokens x 256 weight rows takes two counts (one a CTA of the pair), so narrow tiles can ask for
+// more than there are, and a padded last tile for more partials: the plan passes over the splits that do not fit.
 bool may_split_mn(int M, int N, bool gated, int sms) {
   if (M <= 128 || gated) return false;
   return static_cast<long>((M + 127) / 128) * ((N + 255) / 256) < sms;
@@ -1013,7 +1014,7 @@ qvla_status qvla_debug_set_hooks(unsigned long long wait_limit_ns, int hold_gemm
 qvla_status qvla_debug_gemm_plan(int M, int K, int N, int gated, int sms, int split_room, int* shape, int* parts) {
   g_last_error.clear();
   if (!shape || !parts) return fail(QVLA_ERR_INVALID_ARG, "shape and parts must not be NULL");
-  if (M <= 128) return fail(QVLA_ERR_INVALID_ARG, "M=%d: up to 128 rows run weight-major, not token-major", M);
+  if (M <= 128) return fail(QVLA_ERR_INVALID_ARG, "M=%d: the plan is that of more than 128 rows", M);
   if (K <= 0 || K % 128 != 0) return fail(QVLA_ERR_INVALID_ARG, "K=%d must be a positive multiple of 128", K);
   if (N <= 0 || N % 16 != 0 || (gated && N % 256 != 0))
     return fail(QVLA_ERR_INVALID_ARG, "N=%d must be a positive multiple of 16 (of 256 when gated)", N);
@@ -1033,7 +1034,7 @@ qvla_status qvla_debug_gemm_plan(int M, int K, int N, int gated, int sms, int sp
     a.part_cnt = &no_counts;
     a.part_cnt_n = split_counts_mn(M, N);
   }
-  *shape = qvla::token_major_plan(a, parts);
+  *shape = qvla::gemm_plan(a, parts);
   return QVLA_OK;
 }
 

@@ -100,10 +100,11 @@ struct GemmArgs {
   cudaStream_t stream;
 };
 cudaError_t launch_gemm_w4a4(const GemmArgs& a);
-// The token-major kernel's estimate for int4 activations and M > 128 (host logic only; a's device pointers are not read): the
-// tile shape with the least estimated time (0 single CTAs 128 x 128, 1 single CTAs 128 x 256, 2 CTA pairs 256 x 128, 3 CTA
-// pairs 256 x 256) and *parts, the work units per tile it is estimated with.  The dispatch weighs it against gemm_tmem_plan.
-int token_major_plan(const GemmArgs& a, int* parts);
+// The launch that launch_gemm_w4a4 makes for 4-bit codes, one scale per row and M > 128 (host logic only; a's device pointers
+// are not read): the token-major kernel's tile shape (0 single CTAs 128 x 128, 1 single CTAs 128 x 256, 2 CTA pairs 256 x
+// 128, 3 CTA pairs 256 x 256), or 3 + i for the kernel with the weights in TMEM on tiles of 32 i tokens x 256 weight rows;
+// *parts: work units per tile.
+int gemm_plan(const GemmArgs& a, int* parts);
 
 // The GEMM on CTA pairs with the expanded weights in TMEM (gemm_tmem.cu): operand-byte activations (x_bytes 1 or 2), one
 // scale per row, gated or not.  gemm_tmem_plan (host logic only) picks its tile width *bn (tokens, a multiple of 32) and
