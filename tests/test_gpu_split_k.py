@@ -1,15 +1,13 @@
-"""GPU parity of the token-major GEMM's split of K into work units (Sec. 4.2, Eq. 7).
+"""GPU parity of the GEMM's split of K into work units (csrc/gemm_tmem.cu; Sec. 4.2, Eq. 7).
 
-A non-gated layer whose token-major tiles leave SMs idle splits each tile's k-blocks into 2 or 4
-work units when the caller's workspace has room for their FP32 partials
-(qvla_linear_workspace_bytes counts it); the tile's last unit adds the others' partials to its
-own and applies the epilogue.  Every partial is a non-negative integer multiple of the same power
-of two below 2^24 of them, so the sum is exact in any order: the outputs must be the bits of the
-whole-tile GEMM, which runs when the workspace is one byte short of that room.  Shapes: single
-CTAs with 128- and 256-wide tiles in 4 parts, CTA pairs in 2 parts (the backbone's down
-projection), ragged token and weight edges; a workspace full of garbage (the rotate-quantise
-kernel zeroes the unit counters) and a GEMM run twice after one quantisation (the GEMM leaves
-its counters zero)."""
+A non-gated layer of more than 128 tokens whose tiles leave CTA pairs idle splits each tile's k-blocks into 2 or 4 work
+units when the caller's workspace has room for their FP32 partials (qvla_linear_workspace_bytes counts it); the tile's last
+unit adds the others' partials to its own and applies the epilogue.  Every partial is a non-negative integer multiple of the
+same power of two below 2^24 of them, so the sum is exact in any order: the outputs must be the bits of the whole-tile GEMM,
+which runs when the workspace is one byte short of that room.  Shapes: tiles of 96 to 192 tokens in 2 and 4 parts, one tile
+and many, units of even and odd numbers of k-blocks, ragged token and weight edges (each checked to split by the launch
+plan); the backbone's down projection, which runs whole tiles; a workspace full of garbage (the rotate-quantise kernel zeroes
+the unit counters) and a GEMM run twice after one quantisation (the GEMM leaves its counters zero)."""
 
 import numpy as np
 import pytest
@@ -58,15 +56,23 @@ def _codes_in_workspace(w, M, K):
     return q.reshape(M, K).astype(np.int8), xs, xsum
 
 
-# (M, K, N): single 128-wide tiles in 4 parts with a ragged token tile (150); single 256-wide
-# tiles in 4 parts with a ragged weight tile (300 x 2000); pairs in 2 parts with ragged tokens and
-# weights (700 x 1904); the backbone's down projection (816 x 16384 -> 2048, pairs in 2 parts)
-SPLIT_SHAPES = [(150, 16384, 2048), (256, 16384, 2048), (300, 16384, 2000), (700, 16384, 1904), (816, 16384, 2048)]
+# (M, K, N) and the work units a tile on 152 SMs: a ragged token tile (150), a ragged weight tile (300 x 2000), both (700 x
+# 1904), one tile (129 x 16), units of 27, 28 and 55 k-blocks (K = 14080), and the backbone's down projection in whole tiles
+SPLIT_SHAPES = [(150, 16384, 2048, 4), (256, 16384, 2048, 4), (300, 16384, 2000, 4), (700, 16384, 1904, 2), (129, 16384, 16, 4),
+                (256, 14080, 2048, 4), (400, 14080, 2048, 2), (816, 16384, 2048, 1)]
 
 
-@pytest.mark.parametrize("M,K,N", SPLIT_SHAPES)
-def test_split_equals_whole_tiles(M, K, N):
-    case = W.sweep_linear(M, K, N, seed=M + N, xdtype="bf16", ydtype="bf16", with_bias=True)
+def _check_plan(M, K, N, parts):
+    """The launch on this device splits as the shape is listed for (152 SMs)."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    if sms == 152:
+        assert Q.qvla_debug_gemm_plan(M, K, N, num_sms=sms)[1] == parts
+
+
+@pytest.mark.parametrize("M,K,N,parts", SPLIT_SHAPES)
+def test_split_equals_whole_tiles(M, K, N, parts):
+    _check_plan(M, K, N, parts)
+    case = W.sweep_linear(M, K, N, seed=M + N, xdtype="bf16", ydtype="bf16", had_block=min(2048, K & -K), with_bias=True)
     layer, wq, ws = _layer(case)
     full = Q.qvla_linear_workspace_bytes(layer, M)
     split, work = _linear(layer, case.x, full, with_work=True)
@@ -83,11 +89,12 @@ def test_split_equals_whole_tiles(M, K, N):
     layer.close()
 
 
-def test_split_gemm_twice_after_one_quantisation():
+@pytest.mark.parametrize("M,K,N,parts", [(256, 16384, 2048, 4), (700, 16384, 1904, 2), (400, 14080, 2048, 2)])
+def test_split_gemm_twice_after_one_quantisation(M, K, N, parts):
     """qvla_linear_quantize once, then qvla_linear_gemm twice on the same workspace: the first
     GEMM's last units reset the counters, so the second is the same."""
-    M, K, N = 816, 16384, 2048
-    case = W.sweep_linear(M, K, N, seed=5, xdtype="bf16", ydtype="bf16")
+    _check_plan(M, K, N, parts)
+    case = W.sweep_linear(M, K, N, seed=5, xdtype="bf16", ydtype="bf16", had_block=min(2048, K & -K))
     layer, _, _ = _layer(case)
     nbytes = Q.qvla_linear_workspace_bytes(layer, M)
     work = torch.full((nbytes,), 0x5A, dtype=torch.uint8, device=G.DEV)
