@@ -1,16 +1,14 @@
 // Fused online rotation + symmetric int4 activation quantisation (Sec. 4.1 Eq. 3-5, the online
-// block-Hadamard factor; Sec. 4.2 Eq. 5-6 with per-token or per-step scales).
-//
-// The calibration maxima, and per-step codes in scale groups of 2048 and 4096 channels; every other call takes
-// rotate_quant_wide.cuh or rotate_quant_pass.cu, which share the helpers here.
+// block-Hadamard factor; Sec. 4.2 Eq. 5-6): the calibration maxima, and per-step codes in scale groups of 2048
+// and 4096 channels.  Every other call takes rotate_quant_wide.cuh or rotate_quant_pass.cu, which share the helpers here.
 //
 // One row of x is spread over K/EPT threads, EPT consecutive elements each (16-byte loads),
 // held as float2 pairs.  The fast Walsh-Hadamard transform of a block of b = 2^LOGB elements
 // runs its butterfly stages on the low log2(EPT) index bits in registers (stages of distance
 // >= 2 as packed f32x2 adds/subs), then transposes once through shared memory so that each
 // thread holds the elements that differ in the remaining bits, and runs those in registers
-// too.  The scale (per token: max |y| / 7; or the step's table entry), the codes as operand bytes
-// and the groups' code sums follow from registers.  Instantiated per input dtype in
+// too.  The maximum, or with the step's table entry the codes as operand bytes and the groups' code
+// sums, follow from registers.  Instantiated per input dtype in
 // rotate_quant_{f16,bf16,f32}.cu.
 #pragma once
 
@@ -138,19 +136,17 @@ __device__ __forceinline__ uint32_t sum8_offset(uint32_t w, uint32_t acc) {
 }
 
 // kLogB: log2 of the Hadamard block (0 = no rotation).  kEpt: elements per thread.
-// kStep: the scale is the step table entry (else per token; per-token mode also serves the
-// calibration max when absmax_out is set).  Scale groups: channel k belongs to group
-// k >> gshift (gshift >= 30: one group).  A group holds whole Hadamard blocks and at least 128
-// channels, so all of a thread's elements share one group: with a per-group step table
-// (step_scale[g]) the thread takes its group's entry, xgsum (when set) receives each group's
-// code sum [M][K >> gshift], and calibration (absmax_out) raises one maximum per group.
+// kStep: per-step codes with a scale per channel group; else the calibration maximum.  Scale
+// groups: channel k belongs to group k >> gshift (gshift >= 30: one group, calibration only).  A group
+// holds whole Hadamard blocks and at least 128 channels, so all of a thread's elements share one
+// group: with the per-group step table (step_scale[g]) the thread takes its group's entry, and xgsum
+// receives each group's code sum [M][K >> gshift]; calibration raises absmax_out, one maximum per group.
 template <typename T, int kLogB, int kEpt, bool kStep>
 __global__ void __launch_bounds__(256) rotate_quant_kernel(const T* __restrict__ x, int M, int K, float inv_sqrt_b,
                                                              const float* __restrict__ step_scale,
                                                              uint8_t* __restrict__ xq, float* __restrict__ xscale,
-                                                             int32_t* __restrict__ xsum, float* __restrict__ absmax_out,
-                                                             int gshift, int32_t* __restrict__ xgsum,
-                                                             int32_t* __restrict__ zero, int zero_n) {
+                                                             float* __restrict__ absmax_out, int gshift,
+                                                             int32_t* __restrict__ xgsum) {
   constexpr float kQ = 7.0f;
   constexpr float kBand = kTieBand;
   constexpr int kP = (kEpt == 128) ? 7 : 6;  // log2(kEpt)
@@ -164,8 +160,7 @@ __global__ void __launch_bounds__(256) rotate_quant_kernel(const T* __restrict__
   constexpr int kNV = kEpt / 4;                     // float4 per shared-memory line
 
   extern __shared__ float4 smem4[];
-  __shared__ unsigned int s_max[32];
-  __shared__ unsigned int s_sum[32];
+  __shared__ unsigned int s_max[32];  // calibration
 
   const int tpr = K / kEpt;           // threads per row
   const int rpc = blockDim.x / tpr;   // rows per CTA
@@ -183,15 +178,10 @@ __global__ void __launch_bounds__(256) rotate_quant_kernel(const T* __restrict__
   }
   const int grp = gshift >= 30 ? 0 : e_first >> gshift;
 
-  if (tid < 32) {
-    s_max[tid] = 0u;
-    s_sum[tid] = 0u;
-  }
+  if (!kStep && tid < 32) s_max[tid] = 0u;
 
-  griddep_wait();  // x comes from the previous kernel, which may still read xq / xscale / xsum
+  griddep_wait();  // x comes from the previous kernel, which may still read xq / xscale / xgsum
   griddep_launch_dependents();
-  if (zero != nullptr && blockIdx.x == 0)  // the next GEMM's work-unit counters (its previous use is over)
-    for (int i = tid; i < zero_n; i += blockDim.x) zero[i] = 0;
   float2 v[kN];
   if (active) {
     const T* src = x + static_cast<size_t>(m) * K + static_cast<size_t>(j) * kEpt;
@@ -202,7 +192,7 @@ __global__ void __launch_bounds__(256) rotate_quant_kernel(const T* __restrict__
 #pragma unroll
     for (int i = 0; i < kN; ++i) v[i] = make_float2(0.0f, 0.0f);
   }
-  __syncthreads();  // the reduction slots are cleared before any thread adds to them
+  if constexpr (!kStep) __syncthreads();  // the reduction slots are cleared before any thread raises them
 
   constexpr int kLowBits = kLogB < kP ? kLogB : kP;
   fwht_regs<kN, 0, kLowBits>(v);
@@ -242,16 +232,13 @@ __global__ void __launch_bounds__(256) rotate_quant_kernel(const T* __restrict__
     fwht_regs<kN, kL, kP>(v);
   }
 
-  // ---- scale ----
-  float delta;
-  if constexpr (kStep) {
-    delta = __ldg(step_scale + grp);
-  } else {
+  // ---- calibration: the largest |Z| ----
+  if constexpr (!kStep) {
     float w = 0.0f;
 #pragma unroll
     for (int i = 0; i < kN; ++i) w = fmaxf(w, fmaxf(fabsf(v[i].x), fabsf(v[i].y)));
-    if (absmax_out != nullptr && gshift < 30) {
-      // per-group calibration: the group's threads are consecutive lanes, tg of them (tg | 32)
+    if (gshift < 30) {
+      // per group: the group's threads are consecutive lanes, tg of them (tg | 32)
       const int tg = (1 << gshift) / kEpt;
       for (int o = tg >> 1; o > 0; o >>= 1) w = fmaxf(w, __shfl_xor_sync(0xffffffffu, w, o));
       if (active && (j & (tg - 1)) == 0)
@@ -269,117 +256,86 @@ __global__ void __launch_bounds__(256) rotate_quant_kernel(const T* __restrict__
       atomicMax(&s_max[rloc], __float_as_uint(w));
     }
     __syncthreads();
-    // max |Z| of the normalised rotation: rounding is monotone, so round(max * c) = max round(y * c)
-    const float zmax = __uint_as_float(s_max[rloc]) * inv_sqrt_b;
-    if (absmax_out != nullptr) {  // calibration: one atomic per row
-      if (active && j == 0) atomicMax(reinterpret_cast<unsigned int*>(absmax_out), __float_as_uint(zmax));
-      return;
-    }
-    delta = __fdiv_rn(zmax, kQ);
-  }
-  if (active && j == 0) xscale[m] = delta;
+    // rounding is monotone, so round(max * c) = max round(y * c); one atomic per row
+    if (active && j == 0) atomicMax(reinterpret_cast<unsigned int*>(absmax_out), __float_as_uint(__uint_as_float(s_max[rloc]) * inv_sqrt_b));
+  } else {
+    const float delta = __ldg(step_scale + grp);
+    if (active && j == 0) xscale[m] = delta;
 
-  // ---- codes ----
-  const bool zero_scale = !(delta > 0.0f);
-  const float rcp = zero_scale ? 0.0f : __fdiv_rn(1.0f, delta);
-  const bool tiny_scale = !zero_scale && isinf(rcp);  // 1/delta overflows: plain division
-  const float cr = inv_sqrt_b * rcp;                  // y * cr ~ z / delta (0 when delta = 0: codes 0)
-  // codes in register order, 8 packed nibbles per word (register element r = 8 g + i)
-  uint32_t pk[kEpt / 8];
-  uint32_t sum_acc = 0;
-  const float2 cr2 = make_float2(cr, cr);
-  const float2 magic2 = make_float2(kMagic, kMagic), nmagic2 = make_float2(-kMagic, -kMagic);
-  const float2 neg2 = make_float2(-1.0f, -1.0f);
-#pragma unroll
-  for (int g = 0; g < kEpt / 8; ++g) {
-    // elements 8 g + 2 i (.x) and 8 g + 2 i + 1 (.y), as kMagic + code, two at a time
-    float2 u[4];
-    float dev = 0.0f;  // the largest distance |t - round(t)| of the 8
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      float2 t = __fmul2_rn(v[4 * g + i], cr2);
-      if constexpr (kStep) {
-        t.x = fminf(fmaxf(t.x, -kQ), kQ);
-        t.y = fminf(fmaxf(t.y, -kQ), kQ);
-      }
-      u[i] = __fadd2_rn(t, magic2);
-      const float2 d = __ffma2_rn(__fadd2_rn(u[i], nmagic2), neg2, t);  // t - round(t)
-      dev = fmaxf(dev, fmaxf(fabsf(d.x), fabsf(d.y)));
-    }
-    if (dev >= kBand || tiny_scale) {  // rare: decide these values exactly
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        u[i].x = exact_code(v[4 * g + i].x, inv_sqrt_b, delta, cr, kQ, kBand);
-        u[i].y = exact_code(v[4 * g + i].y, inv_sqrt_b, delta, cr, kQ, kBand);
-      }
-    }
-    // byte j of the packed word: code 8 g + 2 j (low nibble) and 8 g + 2 j + 1 (high nibble)
-    const uint32_t even = low_bytes(u[0].x, u[1].x, u[2].x, u[3].x);
-    const uint32_t odd = low_bytes(u[0].y, u[1].y, u[2].y, u[3].y);
-    pk[g] = (even & 0x0F0F0F0Fu) | ((odd << 4) & 0xF0F0F0F0u);
-    sum_acc = sum8_offset(pk[g], sum_acc);
-  }
-
-  // ---- store: run r holds register elements [r kRun, (r + 1) kRun), contiguous in the row ----
-  if (active) {
-    // One byte per code, the GEMM's tensor-core operand encoding: code q as the E4M3 byte
-    // q + 8 (= q XOR 8).  Within each group of 8 consecutive k the bytes are stored in the order
-    // k0 k2 k4 k6 k1 k3 k5 k7 -- the order the GEMM gives the packed operand it expands -- so
-    // both operands of the dot product agree.
-    uint8_t* dst = xq + static_cast<size_t>(m) * K;
-    uint32_t lo[kEpt / 8], hi[kEpt / 8];
+    // ---- codes ----
+    const bool zero_scale = !(delta > 0.0f);
+    const float rcp = zero_scale ? 0.0f : __fdiv_rn(1.0f, delta);
+    const bool tiny_scale = !zero_scale && isinf(rcp);  // 1/delta overflows: plain division
+    const float cr = inv_sqrt_b * rcp;                  // y * cr ~ z / delta (0 when delta = 0: codes 0)
+    // codes in register order, 8 packed nibbles per word (register element r = 8 g + i)
+    uint32_t pk[kEpt / 8];
+    uint32_t sum_acc = 0;
+    const float2 cr2 = make_float2(cr, cr);
+    const float2 magic2 = make_float2(kMagic, kMagic), nmagic2 = make_float2(-kMagic, -kMagic);
+    const float2 neg2 = make_float2(-1.0f, -1.0f);
 #pragma unroll
     for (int g = 0; g < kEpt / 8; ++g) {
-      lo[g] = (pk[g] ^ 0x88888888u) & 0x0F0F0F0Fu;          // even elements of the 8
-      hi[g] = ((pk[g] >> 4) & 0x0F0F0F0Fu) ^ 0x08080808u;   // odd elements
-    }
+      // elements 8 g + 2 i (.x) and 8 g + 2 i + 1 (.y), as kMagic + code, two at a time
+      float2 u[4];
+      float dev = 0.0f;  // the largest distance |t - round(t)| of the 8
 #pragma unroll
-    for (int run = 0; run < kEpt / kRun; ++run) {
-      int e0;
-      if constexpr (kPhase2) {
-        e0 = ((j >> kR) << kLogB) | (run << kP) | ((j & ((1 << kR) - 1)) << kL);
-      } else {
-        e0 = j * kEpt;
+      for (int i = 0; i < 4; ++i) {
+        float2 t = __fmul2_rn(v[4 * g + i], cr2);
+        t.x = fminf(fmaxf(t.x, -kQ), kQ);
+        t.y = fminf(fmaxf(t.y, -kQ), kQ);
+        u[i] = __fadd2_rn(t, magic2);
+        const float2 d = __ffma2_rn(__fadd2_rn(u[i], nmagic2), neg2, t);  // t - round(t)
+        dev = fmaxf(dev, fmaxf(fabsf(d.x), fabsf(d.y)));
       }
-      uint8_t* gb = dst + (e0 & ~7);  // the 8-byte group this run starts in
-      const int o = e0 & 7;
-      if constexpr (kRun >= 8) {
+      if (dev >= kBand || tiny_scale) {  // rare: decide these values exactly
 #pragma unroll
-        for (int t = 0; t < kRun / 8; ++t) {
-          const int w = run * (kRun / 8) + t;
-          *reinterpret_cast<uint2*>(dst + e0 + 8 * t) = make_uint2(lo[w], hi[w]);
+        for (int i = 0; i < 4; ++i) {
+          u[i].x = exact_code(v[4 * g + i].x, inv_sqrt_b, delta, cr, kQ, kBand);
+          u[i].y = exact_code(v[4 * g + i].y, inv_sqrt_b, delta, cr, kQ, kBand);
         }
-      } else if constexpr (kRun == 4) {  // elements o..o+3 (o = 0 or 4) of a group
-        const int w = run >> 1, h = run & 1;
-        *reinterpret_cast<uint16_t*>(gb + (o >> 1)) = static_cast<uint16_t>(lo[w] >> (16 * h));
-        *reinterpret_cast<uint16_t*>(gb + 4 + (o >> 1)) = static_cast<uint16_t>(hi[w] >> (16 * h));
-      } else {  // kRun == 2: elements o, o+1
-        const int w = run >> 2, q = run & 3;
-        gb[o >> 1] = static_cast<uint8_t>(lo[w] >> (8 * q));
-        gb[4 + (o >> 1)] = static_cast<uint8_t>(hi[w] >> (8 * q));
+      }
+      // byte j of the packed word: code 8 g + 2 j (low nibble) and 8 g + 2 j + 1 (high nibble)
+      const uint32_t even = low_bytes(u[0].x, u[1].x, u[2].x, u[3].x);
+      const uint32_t odd = low_bytes(u[0].y, u[1].y, u[2].y, u[3].y);
+      pk[g] = (even & 0x0F0F0F0Fu) | ((odd << 4) & 0xF0F0F0F0u);
+      sum_acc = sum8_offset(pk[g], sum_acc);
+    }
+
+    // ---- store: run r holds register elements [r kRun, (r + 1) kRun), contiguous in the row ----
+    static_assert(kRun == 2 || kRun == 4, "blocks of 2048 and 4096");
+    if (active) {
+      // One byte per code, the GEMM's tensor-core operand encoding: code q as the E4M3 byte
+      // q + 8 (= q XOR 8).  Within each group of 8 consecutive k the bytes are stored in the order
+      // k0 k2 k4 k6 k1 k3 k5 k7 -- the order the GEMM gives the packed operand it expands -- so
+      // both operands of the dot product agree.
+      uint8_t* dst = xq + static_cast<size_t>(m) * K;
+      uint32_t lo[kEpt / 8], hi[kEpt / 8];
+#pragma unroll
+      for (int g = 0; g < kEpt / 8; ++g) {
+        lo[g] = (pk[g] ^ 0x88888888u) & 0x0F0F0F0Fu;          // even elements of the 8
+        hi[g] = ((pk[g] >> 4) & 0x0F0F0F0Fu) ^ 0x08080808u;   // odd elements
+      }
+#pragma unroll
+      for (int run = 0; run < kEpt / kRun; ++run) {
+        const int e0 = ((j >> kR) << kLogB) | (run << kP) | ((j & ((1 << kR) - 1)) << kL);
+        uint8_t* gb = dst + (e0 & ~7);  // the 8-byte group this run starts in
+        const int o = e0 & 7;
+        if constexpr (kRun == 4) {  // elements o..o+3 (o = 0 or 4) of a group
+          const int w = run >> 1, h = run & 1;
+          *reinterpret_cast<uint16_t*>(gb + (o >> 1)) = static_cast<uint16_t>(lo[w] >> (16 * h));
+          *reinterpret_cast<uint16_t*>(gb + 4 + (o >> 1)) = static_cast<uint16_t>(hi[w] >> (16 * h));
+        } else {  // kRun == 2: elements o, o+1
+          const int w = run >> 2, q = run & 3;
+          gb[o >> 1] = static_cast<uint8_t>(lo[w] >> (8 * q));
+          gb[4 + (o >> 1)] = static_cast<uint8_t>(hi[w] >> (8 * q));
+        }
       }
     }
-  }
-  if (xgsum != nullptr) {  // the code sum of each scale group of the row (tg consecutive lanes)
-    int gs = static_cast<int>(sum_acc) - 8 * kEpt;
+    // the code sum of each scale group of the row (tg consecutive lanes)
+    int gs = static_cast<int>(sum_acc) - 8 * kEpt;  // every code carried an offset
     const int tg = (1 << gshift) / kEpt;
     for (int o = tg >> 1; o > 0; o >>= 1) gs += __shfl_xor_sync(0xffffffffu, gs, o);
     if (active && (j & (tg - 1)) == 0) xgsum[static_cast<size_t>(m) * (K >> gshift) + grp] = gs;
-  }
-  if (xsum != nullptr) {
-    int cs = static_cast<int>(sum_acc) - 8 * kEpt;  // every code carried an offset
-    if ((tpr & 31) == 0) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) cs += __shfl_xor_sync(0xffffffffu, cs, o);
-      if ((tid & 31) == 0) atomicAdd(&s_sum[rloc], static_cast<unsigned int>(cs));
-    } else if ((tpr & (tpr - 1)) == 0) {
-      for (int o = tpr >> 1; o > 0; o >>= 1) cs += __shfl_xor_sync(0xffffffffu, cs, o);
-      if (j == 0) atomicAdd(&s_sum[rloc], static_cast<unsigned int>(cs));
-    } else {
-      atomicAdd(&s_sum[rloc], static_cast<unsigned int>(cs));
-    }
-    __syncthreads();
-    if (active && j == 0) xsum[m] = static_cast<int32_t>(s_sum[rloc]);
   }
 }
 
@@ -421,35 +377,37 @@ cudaError_t launch_t(const RotQuantArgs& a) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   cudaError_t e = cudaLaunchKernelEx(&cfg, kern, reinterpret_cast<const T*>(a.x), a.M, a.K, a.inv_sqrt_b, a.step_scale,
-                                     a.xq, a.xscale, a.xsum, a.mode == 2 ? a.absmax : nullptr,
-                                     a.gshift, a.xgsum, a.zero, a.zero_n);
+                                     a.xq, a.xscale, a.absmax, a.gshift, a.xgsum);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
 
-template <typename T, bool kStep>
-cudaError_t launch_mode(const RotQuantArgs& a) {
-  switch (a.log_b) {
-    case 0: return launch_t<T, 0, kStep>(a);
-    case 1: return launch_t<T, 1, kStep>(a);
-    case 2: return launch_t<T, 2, kStep>(a);
-    case 3: return launch_t<T, 3, kStep>(a);
-    case 4: return launch_t<T, 4, kStep>(a);
-    case 5: return launch_t<T, 5, kStep>(a);
-    case 6: return launch_t<T, 6, kStep>(a);
-    case 7: return launch_t<T, 7, kStep>(a);
-    case 8: return launch_t<T, 8, kStep>(a);
-    case 9: return launch_t<T, 9, kStep>(a);
-    case 10: return launch_t<T, 10, kStep>(a);
-    case 11: return launch_t<T, 11, kStep>(a);
-    case 12: return launch_t<T, 12, kStep>(a);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
 template <typename T>
 cudaError_t launch_dtype(const RotQuantArgs& a) {
-  return a.mode == 1 ? launch_mode<T, true>(a) : launch_mode<T, false>(a);
+  if (a.mode == 1) {  // a group is a Hadamard block there
+    switch (a.log_b) {
+      case 11: return launch_t<T, 11, true>(a);
+      case 12: return launch_t<T, 12, true>(a);
+      default: return cudaErrorInvalidValue;
+    }
+  }
+  if (a.mode != 2) return cudaErrorInvalidValue;
+  switch (a.log_b) {
+    case 0: return launch_t<T, 0, false>(a);
+    case 1: return launch_t<T, 1, false>(a);
+    case 2: return launch_t<T, 2, false>(a);
+    case 3: return launch_t<T, 3, false>(a);
+    case 4: return launch_t<T, 4, false>(a);
+    case 5: return launch_t<T, 5, false>(a);
+    case 6: return launch_t<T, 6, false>(a);
+    case 7: return launch_t<T, 7, false>(a);
+    case 8: return launch_t<T, 8, false>(a);
+    case 9: return launch_t<T, 9, false>(a);
+    case 10: return launch_t<T, 10, false>(a);
+    case 11: return launch_t<T, 11, false>(a);
+    case 12: return launch_t<T, 12, false>(a);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 }  // namespace rq
