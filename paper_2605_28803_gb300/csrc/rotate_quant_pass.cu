@@ -1,14 +1,14 @@
 // Rotate + quantise in passes: the online rotation and activation quantisation (Sec. 4.1 Eq. 3-5,
 // Sec. 4.2 Eq. 5-6) of a few long rows of 16-bit activations into the GEMM's operand bytes, one CTA per
-// 2048-channel pass of a row.
+// pass of 2048 or 1024 channels of a row.
 //
-// The row-per-warp kernel of rotate_quant.cuh gives each thread 64 channels, so a thread's chain
+// The kernel of rotate_quant_wide.cuh gives each thread 32 channels and a row one CTA, so a thread's chain
 // of dependent work is long; with a few rows that chain is the whole kernel.  Here a pass of
-// C channels (C the largest power of two up to 2048 dividing K, holding whole Hadamard blocks) is
+// C channels (2048, or 1024 where that does not divide K, holding whole Hadamard blocks) is
 // spread over 256 threads, 8 channels each: the butterflies on index bits 0-2 run in registers,
 // on bits 3-7 across the lanes, and after one transpose through shared memory thread t holds the
 // channels t + 256 w (w < 8) and runs bits 8-10.  The stage order and every rounding are those of
-// the row-per-warp kernel (stages in increasing index-bit order, each sum and difference rounded
+// that kernel (stages in increasing index-bit order, each sum and difference rounded
 // once), and so are the scale and the codes (its fast path, tie band and exact rule, value by
 // value), so the outputs are the same bits.  The P = K / C passes of a row form a cluster: with
 // per-token scales each CTA sends its pass's largest |value| to every CTA of the cluster
@@ -26,7 +26,7 @@ constexpr int kRqpThreads = 256;
 // test hook (qvla_debug.h): nonzero, the CTAs of a cluster send each other nothing, so every
 // receiving wait runs out
 static __device__ int g_rqp_hold;
-constexpr int kRqpMaxPasses = 8;  // a cluster of at most 8 CTAs (K <= 16384)
+constexpr int kRqpMaxPasses = 8;  // a cluster of 3 to 8 CTAs
 constexpr int kRqpMaxRows = 48;   // the rows it takes, of more than kRqpMinK channels
 constexpr int kRqpMinK = 4096;
 
@@ -53,19 +53,16 @@ __global__ void __launch_bounds__(kRqpThreads) rotate_quant_pass_kernel(RqpParam
   uint8_t* const s_out = smem + 4 * C;                  // [C] its operand bytes
   const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   const int m = static_cast<int>(blockIdx.x) / P, rank = static_cast<int>(blockIdx.x) % P;
-  const bool exch_max = !kStep && P > 1;
-  const bool hold = P > 1 && *const_cast<volatile int*>(&g_rqp_hold) != 0;
-  if (P > 1) {
-    // the cluster barrier completed before the first send guarantees every receiver's barrier
-    if (t == 0) {
-      mbar_init(smem_u32(&bar_max), 1);
-      mbar_init(smem_u32(&bar_sum), 1);
-      mbar_init_fence();
-      if (exch_max) mbar_arrive_expect_tx(smem_u32(&bar_max), static_cast<uint32_t>(4 * P));
-      if (rank == 0) mbar_arrive_expect_tx(smem_u32(&bar_sum), static_cast<uint32_t>(4 * P));
-    }
-    cluster_arrive_relaxed();
+  const bool hold = *const_cast<volatile int*>(&g_rqp_hold) != 0;
+  // the cluster barrier completed before the first send guarantees every receiver's barrier
+  if (t == 0) {
+    mbar_init(smem_u32(&bar_max), 1);
+    mbar_init(smem_u32(&bar_sum), 1);
+    mbar_init_fence();
+    if (!kStep) mbar_arrive_expect_tx(smem_u32(&bar_max), static_cast<uint32_t>(4 * P));
+    if (rank == 0) mbar_arrive_expect_tx(smem_u32(&bar_sum), static_cast<uint32_t>(4 * P));
   }
+  cluster_arrive_relaxed();
   griddep_wait();  // x comes from the previous kernel, which may still read xq / xscale / xsum
   griddep_launch_dependents();
   if (p.zero != nullptr && blockIdx.x == 0)  // the next GEMM's work-unit counters
@@ -143,8 +140,8 @@ __global__ void __launch_bounds__(kRqpThreads) rotate_quant_pass_kernel(RqpParam
 #pragma unroll
   for (int i = 0; i < kRqpThreads / 32; ++i) cmax = max(cmax, s_wmax[i]);
   bool ok = true;
-  if (P > 1) cluster_wait();  // pairs with the arrive at set-up
-  if (exch_max) {
+  cluster_wait();  // pairs with the arrive at set-up
+  if (!kStep) {
     if (t < P && !hold)
       st_async_u32(mapa_shared(smem_u32(&s_maxes[rank]), static_cast<uint32_t>(t)), cmax,
                    mapa_shared(smem_u32(&bar_max), static_cast<uint32_t>(t)));
@@ -164,7 +161,7 @@ __global__ void __launch_bounds__(kRqpThreads) rotate_quant_pass_kernel(RqpParam
     const int e = t + 256 * w;
     if (e < C) {
       const float y = yv[w];
-      float tt = __fmul_rn(y, cr);  // rounded on its own, as the row-per-warp kernel's packed multiply
+      float tt = __fmul_rn(y, cr);  // rounded on its own, as the other kernel's packed multiply
       if (kStep) tt = fminf(fmaxf(tt, -7.0f), 7.0f);
       float u = __fadd_rn(tt, rq::kMagic);
       const float d = __fmaf_rn(__fadd_rn(u, -rq::kMagic), -1.0f, tt);
@@ -185,14 +182,12 @@ __global__ void __launch_bounds__(kRqpThreads) rotate_quant_pass_kernel(RqpParam
   uint32_t csum = 0u;
 #pragma unroll
   for (int i = 0; i < kRqpThreads / 32; ++i) csum += s_wsum[i];
-  if (P > 1) {
-    if (t == 0 && !hold)
-      st_async_u32(mapa_shared(smem_u32(&s_sums[rank]), 0u), csum, mapa_shared(smem_u32(&bar_sum), 0u));
-    if (rank == 0) {
-      ok = mbar_wait_cluster(smem_u32(&bar_sum), 0) && ok;
-      csum = 0u;
-      for (int src = 0; src < P; ++src) csum += s_sums[src];
-    }
+  if (t == 0 && !hold)
+    st_async_u32(mapa_shared(smem_u32(&s_sums[rank]), 0u), csum, mapa_shared(smem_u32(&bar_sum), 0u));
+  if (rank == 0) {
+    ok = mbar_wait_cluster(smem_u32(&bar_sum), 0) && ok;
+    csum = 0u;
+    for (int src = 0; src < P; ++src) csum += s_sums[src];
   }
   (void)ok;  // a wait that ran out has recorded QVLA_ERR_TIMEOUT; the outputs are then not defined
   if (rank == 0 && t == 0) {
@@ -217,7 +212,7 @@ cudaError_t launch_rqp(const RotQuantArgs& a, const RqpParams& p) {
   attr[1].val.clusterDim.y = 1;
   attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = p.P > 1 ? 2 : 1;
+  cfg.numAttrs = 2;
   cudaError_t e = cudaLaunchKernelEx(&cfg, kern, p);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
@@ -235,10 +230,9 @@ cudaError_t launch_rotate_quant_pass(const RotQuantArgs& a, bool* launched) {
   if (a.out_mode != 1 || (a.mode != 0 && a.mode != 1) || (a.xdt != 0 && a.xdt != 1) || a.gshift < 30 ||
       a.xgsum != nullptr || a.M < 1 || a.M > kRqpMaxRows || a.K <= kRqpMinK)
     return cudaSuccess;
-  int C = 2048;
-  while (a.K % C != 0) C /= 2;
+  const int C = a.K % 2048 == 0 ? 2048 : 1024;
   const int P = a.K / C;
-  if (a.log_b < 0 || (1 << a.log_b) > C || P > kRqpMaxPasses || C < 128) return cudaSuccess;
+  if (a.K % C != 0 || a.log_b < 0 || (1 << a.log_b) > C || P > kRqpMaxPasses) return cudaSuccess;
   RqpParams p;
   p.x = a.x;
   p.xq = a.xq;
