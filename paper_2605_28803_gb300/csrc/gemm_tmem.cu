@@ -29,11 +29,11 @@
 // k-blocks are filled and released one by one, which hides the release-refill latency (about 1400 cycles) at bn = 192,
 // where the ring holds four k-blocks.
 //
-// GEMM alone, in us, token-major kernel before and this one: 816 x 2048 -> 2 x 16384 gated 60.4 and 41.1 (2660 TFLOP/s
+// GEMM alone, in us, token-major kernel before and this one: 816 x 2048 -> 2 x 16384 gated 60.4 and 42.3 (2590 TFLOP/s
 // of the integer product); 816 x 16384 -> 2048 38.0 and 26.9; 8192 x 2048 -> 16384 240 and 146 (3770 TFLOP/s); 3200 x
-// 16384 -> 2048 104.6 and 58.4 (3680 TFLOP/s); 8-bit codes, 816 x 2048 -> 2 x 16384 gated 79 and 61.  Packed 4-bit codes,
+// 16384 -> 2048 104.6 and 58.4 (3680 TFLOP/s); 8-bit codes, 816 x 2048 -> 2 x 16384 gated 79 and 63.  Packed 4-bit codes,
 // expanded by the converters next to the weights: 777 x 4096 -> 1024 18.0 and 12.5, 5781 x 3712 -> 7392 142 and 121, 816 x
-// 2048 -> 2 x 16384 gated 72 and 57, 50 x 2048 -> 2 x 4096 gated 15.1 and 8.1; a k-block costs the converters 235 to 290 ns
+// 2048 -> 2 x 16384 gated 72 and 59, 50 x 2048 -> 2 x 4096 gated 15.1 and 7.9; a k-block costs the converters 235 to 290 ns
 // there (the codes fetched before the wait for the TMEM stage, and the proxy fence moved up to the stores, were slower: 40
 // against 34 us at 200 x 16384 -> 2048).  Bound now by the
 // issue round of the MMA warp (about 430 cycles a k-block up to bn = 160) and the refill of the TMEM stages (about 470 at
@@ -47,7 +47,8 @@ constexpr int kTmEpiWarps = 8, kTmConv = 8, kTmMma = 24, kTmTmaX = 25, kTmTmaW =
 constexpr int kTmGroups = 4;  // converter groups
 constexpr int kTmEpiThreads = kTmEpiWarps * 32;
 constexpr int kTmThreads = 28 * 32;
-// Registers: 72 a thread at launch (896 x 72 = 64512); the roles then take 256 x 120 + 512 x 56 + 128 x 40 = 64512.
+// Registers: 72 a thread at launch (896 x 72 = 64512); the roles then take 256 x 120 + 512 x 56 + 128 x 40 = 64512.  The
+// instances for operand bytes of 4-bit codes spill 6 bytes a thread (-Xptxas -v), the others none.
 constexpr int kTmRegsEpi = 120, kTmRegsConv = 56, kTmRegsOther = 40;
 static_assert(256 * kTmRegsEpi + 512 * kTmRegsConv + 128 * kTmRegsOther <= kTmThreads * 72, "register split");
 constexpr int kTmMaxBn = 192;          // 2 x 192 accumulator columns leave two weight stages of two k-blocks
@@ -696,8 +697,8 @@ cudaError_t launch_tm(const GemmArgs& a, int bn, int parts) {
   return cudaGetLastError();
 }
 
-// Estimated time (ns) of a launch with tiles of bn tokens in `parts` work units, fitted to GB300 measurements (M 5-8192,
-// K 128-16384, N 16-32768; over 1876 shapes within 16%, half of them within 3%): a fixed cost, more with more pairs at
+// Estimated time (ns) of a launch with tiles of bn tokens in `parts` work units, fitted to GB300 measurements (1876 launches,
+// M 5-1500, K 128-16384, weight rows 16-32768: within 16%, half of them within 4%): a fixed cost, more with more pairs at
 // work, with the last tile's epilogue; the first unit's k-blocks (165 ns each up to bn = 128, 172 at 160, 200 at 192; two
 // planes 250, or 1.95 bn; packed codes 235 to 290); per further wave of pairs a unit's k-blocks and hand-over, or the epilogue where that is
 // longer; with K split, the partial's write and read-back.

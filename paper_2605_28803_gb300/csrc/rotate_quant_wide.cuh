@@ -3,7 +3,8 @@
 //
 // It does what rotate_quant.cuh's kernel does, bit for bit, with fewer instructions
 // per channel and twice the warps in flight:
-//   * a thread holds 32 channels instead of 64: 64 registers, 32 warps per SM;
+//   * a thread holds 32 channels instead of 64: 64 registers, 32 warps per SM.  (19 of the 312 instances, all with a scale per
+//     step, spill 4 to 24 bytes a thread there, most with blocks of 512: -Xptxas -v);
 //   * the butterflies run in three phases, index bits 0-4 on 32 consecutive channels, 5-7 (5-6 among 4 threads for blocks of
 //     64 and 128, whose rows need not be whole 256-channel groups), and 8-10 (8-11 for blocks of 4096, on half quads), with a transpose through shared memory between phases whose stores and loads both move 16
 //     bytes (4 channels, a quad) per thread.  A quad is the channels whose codes fill one 32-bit word of the output, so after the last phase every code leaves in a
