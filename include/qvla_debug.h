@@ -45,6 +45,11 @@ qvla_status qvla_debug_set_hooks(unsigned long long wait_limit_ns, int hold_gemm
  * positive multiple of 128, N not a positive multiple of 16 (256 when gated), num_sms < 2. */
 qvla_status qvla_debug_gemm_plan(int M, int K, int N, int gated, int num_sms, int split_room, int* shape, int* parts);
 
+/* The same for the other activations: codes 0, packed 4-bit codes (qvla_gemm_w4a4); 1,
+ * qvla_w4a4_linear's; 2, 8-bit codes (qvla_w4a8_linear, qvla_gemm_w4a8).  Only 1 splits K. */
+qvla_status qvla_debug_gemm_plan_codes(int codes, int M, int K, int N, int gated, int num_sms, int split_room, int* shape,
+                                       int* parts);
+
 #ifdef __cplusplus
 }
 #endif

@@ -1012,7 +1012,12 @@ qvla_status qvla_debug_set_hooks(unsigned long long wait_limit_ns, int hold_gemm
 }
 
 qvla_status qvla_debug_gemm_plan(int M, int K, int N, int gated, int sms, int split_room, int* shape, int* parts) {
+  return qvla_debug_gemm_plan_codes(1, M, K, N, gated, sms, split_room, shape, parts);
+}
+
+qvla_status qvla_debug_gemm_plan_codes(int codes, int M, int K, int N, int gated, int sms, int split_room, int* shape, int* parts) {
   g_last_error.clear();
+  if (codes < 0 || codes > 2) return fail(QVLA_ERR_INVALID_ARG, "codes=%d must be 0, 1 or 2", codes);
   if (!shape || !parts) return fail(QVLA_ERR_INVALID_ARG, "shape and parts must not be NULL");
   if (M <= 128) return fail(QVLA_ERR_INVALID_ARG, "M=%d: the plan is that of more than 128 rows", M);
   if (K <= 0 || K % 128 != 0) return fail(QVLA_ERR_INVALID_ARG, "K=%d must be a positive multiple of 128", K);
@@ -1020,7 +1025,7 @@ qvla_status qvla_debug_gemm_plan(int M, int K, int N, int gated, int sms, int sp
     return fail(QVLA_ERR_INVALID_ARG, "N=%d must be a positive multiple of 16 (of 256 when gated)", N);
   if (sms < 2) return fail(QVLA_ERR_INVALID_ARG, "num_sms=%d must be at least 2", sms);
   qvla::GemmArgs a = {};
-  a.x_bytes = 1;
+  a.x_bytes = codes;
   a.M = M;
   a.N = N;
   a.K = K;
@@ -1028,7 +1033,7 @@ qvla_status qvla_debug_gemm_plan(int M, int K, int N, int gated, int sms, int sp
   a.num_sms = sms;
   static float no_floats;  // stand-ins for the workspace: the plan reads only whether it is there
   static int no_counts;
-  if (split_room && may_split_mn(M, N, gated != 0, sms)) {
+  if (codes == 1 && split_room && may_split_mn(M, N, gated != 0, sms)) {
     a.part_ws = &no_floats;
     a.part_ws_floats = split_floats_mn(M, N);
     a.part_cnt = &no_counts;

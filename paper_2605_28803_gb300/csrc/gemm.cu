@@ -53,7 +53,7 @@ TileShape token_major_shape(const GemmArgs& a, long* estimate = nullptr) {
 }
 
 // Whether the kernel with the weights in TMEM takes the launch, with its plan.  From K = 768 it was faster than the
-// token-major kernel at every shape measured (M 129-8192 and gated M 5-128, N 16-32768: 1.05 to 2.8 times); below, the
+// token-major kernel at every shape measured (M 129-8192 and gated M 5-128, N 16-32768: 1.04 to 2.8 times); below, the
 // estimates decide.  Up to 128 tokens a layer that is not gated keeps the weight-major kernel: alone the other is faster
 // from K N = 2^21 or so, but between the small kernels of a chain it is not (the action head's step at 50 tokens: 240
 // against 221 us), as its pairs fill the SMs' shared memory and TMEM and so start late.  Packed 4-bit codes go by the estimates
@@ -70,19 +70,23 @@ bool take_tmem(const GemmArgs& a, int* bn, int* parts) {
   return t < old;
 }
 
+// 8-bit activation planes on single CTAs: whether 128-wide tiles beat 256-wide ones, by waves x tile width (a gated layer's
+// gate and up rows share a 256-row tile).
+bool a8_narrow(const GemmArgs& a) {
+  const long tm = (a.M + kBM - 1) / kBM;
+  const long w256 = (tm * ((a.N + 255) / 256) + a.num_sms - 1) / a.num_sms;
+  const long w128 = (tm * ((a.N + 127) / 128) + a.num_sms - 1) / a.num_sms;
+  return !a.gated && w128 * 128 < w256 * 256;
+}
+
 template <int kX, typename OutT>
 cudaError_t launch_out(const GemmArgs& a) {
   int bn = 0, parts = 1;
   if (take_tmem(a, &bn, &parts)) return launch_gemm_tmem(a, bn, parts);
   if (a.gated || a.M > 128) {
     if constexpr (kX == 2) {
-      // 8-bit activation planes: single CTAs; tile width by waves x tile width
-      if (a.gated) return launch_cfg<256, false, true, kX, OutT>(a);  // gate/up pairs share a 256-row tile
-      const long tm = (a.M + kBM - 1) / kBM;
-      const long w256 = (tm * ((a.N + 255) / 256) + a.num_sms - 1) / a.num_sms;
-      const long w128 = (tm * ((a.N + 127) / 128) + a.num_sms - 1) / a.num_sms;
-      if (w128 * 128 < w256 * 256) return launch_cfg<128, false, false, kX, OutT>(a);
-      return launch_cfg<256, false, false, kX, OutT>(a);
+      if (a.gated) return launch_cfg<256, false, true, kX, OutT>(a);
+      return a8_narrow(a) ? launch_cfg<128, false, false, kX, OutT>(a) : launch_cfg<256, false, false, kX, OutT>(a);
     } else {
       // gated layers always take 256-wide tiles: a tile's gate and up rows meet in one epilogue.  Operand bytes come here
       // below K = 768 only, where no pairs are planned.
@@ -111,6 +115,7 @@ int gemm_plan(const GemmArgs& a, int* parts) {
   *parts = 1;
   if (take_tmem(a, &bn, parts)) return 3 + bn / 32;
   *parts = 1;
+  if (a.x_bytes == 2) return static_cast<int>(a8_narrow(a) ? TileShape::kSingle128 : TileShape::kSingle256);
   return static_cast<int>(token_major_shape(a));
 }
 

@@ -100,8 +100,8 @@ struct GemmArgs {
   cudaStream_t stream;
 };
 cudaError_t launch_gemm_w4a4(const GemmArgs& a);
-// The launch that launch_gemm_w4a4 makes for 4-bit codes, one scale per row and M > 128 (host logic only; a's device pointers
-// are not read): the token-major kernel's tile shape (0 single CTAs 128 x 128, 1 single CTAs 128 x 256, 2 CTA pairs 256 x
+// The launch that launch_gemm_w4a4 makes for one scale per row and M > 128 (host logic only; a's device pointers are not
+// read): the token-major kernel's tile shape (0 single CTAs 128 x 128, 1 single CTAs 128 x 256, 2 CTA pairs 256 x
 // 128, 3 CTA pairs 256 x 256), or 3 + i for the kernel with the weights in TMEM on tiles of 32 i tokens x 256 weight rows;
 // *parts: work units per tile.
 int gemm_plan(const GemmArgs& a, int* parts);

@@ -57,6 +57,7 @@ SIGNATURES = {
     "qvla_check_device": (_I, [_P]),
     "qvla_debug_set_hooks": (_I, [ctypes.c_ulonglong, _I]),
     "qvla_debug_gemm_plan": (_I, [_I, _I, _I, _I, _I, _I, _P, _P]),
+    "qvla_debug_gemm_plan_codes": (_I, [_I, _I, _I, _I, _I, _I, _I, _P, _P]),
 }
 
 
@@ -315,4 +316,13 @@ def qvla_debug_gemm_plan(M: int, K: int, N: int, gated: bool = False, num_sms: i
     shape, parts = ctypes.c_int(-1), ctypes.c_int(0)
     _check(_lib.qvla_debug_gemm_plan(M, K, N, 1 if gated else 0, num_sms, 1 if split_room else 0,
                                      ctypes.addressof(shape), ctypes.addressof(parts)))
+    return GEMM_SHAPES[shape.value], parts.value
+
+
+def qvla_debug_gemm_plan_codes(codes: int, M: int, K: int, N: int, gated: bool = False, num_sms: int = 152,
+                               split_room: bool = True) -> tuple[str, int]:
+    """The same for packed 4-bit codes (0), qvla_w4a4_linear's activations (1) or 8-bit codes (2)."""
+    shape, parts = ctypes.c_int(-1), ctypes.c_int(0)
+    _check(_lib.qvla_debug_gemm_plan_codes(codes, M, K, N, 1 if gated else 0, num_sms, 1 if split_room else 0,
+                                           ctypes.addressof(shape), ctypes.addressof(parts)))
     return GEMM_SHAPES[shape.value], parts.value

@@ -1,8 +1,9 @@
 """GPU parity of the int4 x int4 GEMM and its dequantisation epilogue (Sec. 4.2, Eq. 7).
 
-G2: on the oracle's codes the int32 accumulator is bit-exact for every tile shape, ragged M and
-N edges and both orientations (tokens on the MMA's M side for M > 128, weights otherwise),
-including the weight-major split of K over clusters of 2, 4 and 8 CTAs.
+G2: on the oracle's codes the int32 accumulator is bit-exact with ragged M and N edges, on the
+weight-major kernel up to 128 tokens, including its split of K over clusters of 2, 4 and 8 CTAs, and
+above on the CTA-pair kernel with the weights in TMEM, at every tile width, and the token-major one
+(1000 x 128 -> 2048 and 2048 x 256 -> 4096; its other tile shapes are in test_gpu_token_major.py).
 G3: the E4M3 / FP32 tensor-core path stays exact at the largest sums K = 16384 allows.
 G5: outputs within 2e-3 of the tensor's maximum magnitude."""
 
@@ -42,12 +43,10 @@ def _run(M, N, K, seed, ydt="f16", with_bias=True):
     # weight-major split-K: a cluster of 2 with several reduction elements per thread, 5
     # k-blocks over 4 CTAs (uneven slices) with a ragged weight tile, a decode row at K = 16384
     (100, 8192, 1024), (33, 400, 640), (1, 2048, 16384),
-    # token-major at larger M: 128- and 256-wide tiles with ragged last token tiles (1100, 1450)
-    # beside a ragged weight tile, and several tiles per persistent CTA (640 x 16384)
+    # larger M: ragged last token tiles (1100, 1450) beside a ragged weight tile, and several tiles per
+    # persistent CTA (640 x 16384)
     (1024, 384, 1024), (1100, 1008, 512), (1450, 2048, 1024), (2048, 4096, 256), (640, 16384, 2048),
-    # CTA pairs (256-token tiles over two SMs, 128- and 256-wide): the last tile's second CTA
-    # without tokens beside a ragged weight tile (600 x 8432, 260 x 13264), a ragged second CTA
-    # (1450), several pair tiles per CTA (640 x 16384 above); the backbone's down projection
+    # wide layers with ragged weight tiles (600 x 8432, 260 x 13264); the backbone's down projection
     (600, 8432, 1024), (1450, 4352, 1024), (260, 13264, 1024), (816, 2048, 16384),
 ])
 def test_gemm_accumulator_bit_exact(M, N, K):
@@ -103,11 +102,9 @@ def test_gemm_zero_scale_gives_bias():
 @pytest.mark.parametrize("M,H,K", [(512, 128, 256), (600, 256, 512), (1450, 384, 1024), (520, 4096, 1024),
                                    (1450, 4224, 1024)])
 def test_gated_gemm_bit_exact(M, H, K):
-    """Gated layers (gate and up rows of a hidden unit in one 256-wide tile): [gate | up]
-    accumulators bit-exact and h = gelu(gate) * up within the output tolerance, with ragged
-    last token tiles (600, 1450) and a ragged tile of hidden units (H = 384); the two larger
-    cases run on CTA pairs, the gate rows staged by one CTA and the up rows by the other, with
-    the last tile's second CTA without tokens (520) or ragged (1450)."""
+    """Gated layers (gate and up rows of a hidden unit in one tile): [gate | up] accumulators
+    bit-exact and h = gelu(gate) * up within the output tolerance, with ragged last token tiles
+    (600, 1450, 520), H = 384 and several tiles a CTA pair."""
     rng = np.random.default_rng(M + H + K)
     qx = _codes(rng, M, K, -7, 7)
     qg, qu = _codes(rng, H, K), _codes(rng, H, K)

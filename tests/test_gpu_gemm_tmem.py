@@ -3,7 +3,8 @@
 qvla_w4a4_linear's GEMM takes it for batches of more than 128 tokens and for gated layers from 5 (below K = 768 where it is
 estimated faster); qvla_gemm_w4a4 takes packed codes there where it is estimated faster, else to the token-major kernel, and
 expands them in its converters.  Every accumulation is exact and the epilogue is the same operations, so the outputs must be
-the same bits, also of slices of a few tokens, which run the weight-major kernel and the GEMV.  Shapes sit at the edges of its tiles: one k-block and odd counts of them (the last ring stage holds one), token
+the same bits as on packed codes and as those of slices of a few tokens, which run the weight-major kernel and, gated, the GEMV.
+Shapes sit at the edges of its tiles: one k-block and odd counts of them (the last ring stage holds one), token
 counts around the tile widths, weight rows past 64-, 128- and 256-row boundaries, tiles in several waves, K split into work
 units, and gated layers from a few tokens.  With 8-bit codes the accumulators must be the oracle's integers."""
 
@@ -48,6 +49,17 @@ def _both(layer, x, M, dt):
     return y, ref
 
 
+def _equal_slices(layer, x, y, rows):
+    """The linear on slices of `rows` tokens, in other kernels, gives the same bits."""
+    work = torch.empty(Q.qvla_linear_workspace_bytes(layer, rows), dtype=torch.uint8, device=G.DEV)
+    for i in range(0, x.shape[0], rows):
+        m = min(rows, x.shape[0] - i)
+        part = torch.full((m, layer.N), float("nan"), dtype=y.dtype, device=G.DEV)
+        Q.qvla_w4a4_linear(layer, x[i:], m, -1, part, work, work.numel(), G.stream())
+        assert torch.equal(y[i : i + m], part)
+    Q.qvla_check_device(G.stream())
+
+
 @pytest.mark.parametrize("M,K,N,dt", [
     (129, 768, 16, "f16"), (160, 896, 272, "bf16"), (191, 1152, 528, "f16"), (192, 1024, 1040, "bf16"),
     (193, 2176, 1552, "f16"), (385, 1152, 4096, "bf16"), (2500, 1024, 2560, "f16"), (1500, 128, 4112, "bf16"),
@@ -58,17 +70,19 @@ def test_equals_the_other_kernels_bit_for_bit(M, K, N, dt):
     x = torch.from_numpy(rng.standard_normal((M, K), dtype=np.float32)).to(_T[dt]).to(G.DEV)
     y, ref = _both(layer, x, M, dt)
     assert torch.equal(y, ref)
+    _equal_slices(layer, x, y, 128)
     layer.close()
 
 
 @pytest.mark.parametrize("M,K,H,dt", [(5, 128, 128, "bf16"), (33, 640, 256, "f16"), (128, 1152, 384, "bf16"),
                                       (130, 896, 384, "f16"), (816, 2048, 1024, "bf16"), (1000, 768, 8192, "f16")])
-def test_gated_equals_the_token_major_kernel(M, K, H, dt):
+def test_gated_equals_packed_codes_and_slices(M, K, H, dt):
     rng = np.random.default_rng(M + K + H)
     layer, _ = _layer(rng, H, K, 64, dt, gated=True)
     x = torch.from_numpy(rng.standard_normal((M, K), dtype=np.float32)).to(_T[dt]).to(G.DEV)
     y, ref = _both(layer, x, M, dt)
     assert torch.equal(y, ref)
+    _equal_slices(layer, x, y, 4)
     layer.close()
 
 

@@ -5,8 +5,8 @@ limit to 20 ms, so the converters' waits for the staged tiles, the MMA thread's 
 expanded tiles and the epilogue's wait for the accumulator all run out.  The kernel must record
 QVLA_ERR_TIMEOUT, issue no MMA, leave the output untouched and return; qvla_check_device reports
 it once and clears it, and the next launch is bit-exact.  The held kernel has no copy, MMA or
-asynchronous store outstanding when it returns (it is the token-major single-CTA form: no cluster
-exchange), so nothing faults or hangs."""
+asynchronous store outstanding when it returns (no form here exchanges data in a cluster), so nothing
+faults or hangs."""
 
 import numpy as np
 import pytest
@@ -19,11 +19,13 @@ from tests import gpu_helpers as G
 pytestmark = pytest.mark.gpu
 
 
-def test_a_wait_that_runs_out_reports_timeout_and_the_next_launch_is_clean():
+@pytest.mark.parametrize("M,K,N,kernel", [(256, 512, 256, "tmem 32x256"), (405, 1152, 4800, "single 128x128")])
+def test_a_wait_that_runs_out_reports_timeout_and_the_next_launch_is_clean(M, K, N, kernel):
+    """Packed codes on the CTA-pair kernel with the weights in TMEM and on the token-major kernel."""
+    assert Q.qvla_debug_gemm_plan_codes(0, M, K, N, num_sms=152) == (kernel, 1)
     rng = np.random.default_rng(61)
-    M, K, N = 256, 512, 256
     wcodes = rng.integers(-7, 8, (N, K)).astype(np.int8)
-    layer = G.make_layer(O.pack_int4(wcodes), np.full(N, 0.01, np.float32), 512, "f16", "f16")
+    layer = G.make_layer(O.pack_int4(wcodes), np.full(N, 0.01, np.float32), 128, "f16", "f16")
     xcodes = rng.integers(-7, 8, (M, K)).astype(np.int8)
     xq, xs = O.pack_int4(xcodes), np.full(M, 0.02, np.float32)
     xsum = xcodes.astype(np.int64).sum(1)
