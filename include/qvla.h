@@ -207,7 +207,8 @@ qvla_status qvla_layer_info(const qvla_layer* layer, int* N, int* K, int* had_bl
  *   step == -1 : per-token scale xscale[m] = max_k |y_k| / 7               (backbone)
  *   step >= 0  : xscale[m] = table[step] of the layer                        (DiT, Eq. 6)
  * and codes clamp(round(y / xscale[m]), -7, 7), round half to even on the exact quotient of
- * the float32 operands; xscale = 0 gives codes 0.
+ * the float32 operands; xscale = 0 gives codes 0.  A NaN anywhere in row m makes its per-token scale NaN
+ * (its codes then carry nothing), and so the linear's row m of y; a per-step scale clamps a NaN.
  *   xq      device out [M][K/2] packed codes.     xscale device out [M] float32.
  *   xsum    device out [M] int32 (may be NULL): sum over k of the codes of row m.  The GEMM
  *           needs it (its operand encoding is offset binary; the sum removes the offset).

@@ -30,8 +30,8 @@
 // where the ring holds four k-blocks.
 //
 // GEMM alone, in us, token-major kernel before and this one: 816 x 2048 -> 2 x 16384 gated 60.4 and 42.3 (2590 TFLOP/s
-// of the integer product); 816 x 16384 -> 2048 38.0 and 26.9; 8192 x 2048 -> 16384 240 and 146 (3770 TFLOP/s); 3200 x
-// 16384 -> 2048 104.6 and 58.4 (3680 TFLOP/s); 8-bit codes, 816 x 2048 -> 2 x 16384 gated 79 and 63.  Packed 4-bit codes,
+// of the integer product); 816 x 16384 -> 2048 38.0 and 26.2; 8192 x 2048 -> 16384 240 and 146 (3770 TFLOP/s); 3200 x
+// 16384 -> 2048 104.6 and 57.4 (3740 TFLOP/s); 8-bit codes, 816 x 2048 -> 2 x 16384 gated 79 and 63.  Packed 4-bit codes,
 // expanded by the converters next to the weights: 777 x 4096 -> 1024 18.0 and 12.5, 5781 x 3712 -> 7392 142 and 121, 816 x
 // 2048 -> 2 x 16384 gated 72 and 59, 50 x 2048 -> 2 x 4096 gated 15.1 and 7.9; a k-block costs the converters 235 to 290 ns
 // there (the codes fetched before the wait for the TMEM stage, and the proxy fence moved up to the stores, were slower: 40

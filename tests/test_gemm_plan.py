@@ -3,7 +3,7 @@ takes for M > 128 tokens, read through qvla_debug_gemm_plan (host logic only, no
 
 The plan is a launch-time estimate fitted to GB300 measurements; these tests pin the decisions the measurements justified and
 the rules around them:
-  * the backbone's down projection (816 x 16384 -> 2048) runs CTA pairs on whole 128-token tiles, the weights in TMEM (26.9 us
+  * the backbone's down projection (816 x 16384 -> 2048) runs CTA pairs on whole 128-token tiles, the weights in TMEM (26.2 us
     against 38.0 for the token-major kernel's CTA pairs with K in 2 work units);
   * few tiles of many k-blocks split: 256 x 16384 -> 2048 into 4 units;
   * from K = 768 every launch takes that kernel; below, the estimates weigh it against the token-major kernel;
